@@ -19,11 +19,15 @@
 //    pairs, same rounding per pair as nb_pair). The kernel is bound by
 //    instruction issue, and packing halves the issue slots of the FP32 work.
 //  - j data (coordinates and charge, type, mask word) of group g + 1 are
-//    copied into shared memory with cp.async from the start of group g
-//    (their slot words were loaded one group earlier still); the
-//    shift vectors come from a per-warp shared copy of the system's 27; the
-//    row pairs' positions and charges and their LJ coefficients by j type
-//    sit in per-warp shared tables, already in packed order.
+//    loaded into registers while group g is computed, their slot words one
+//    group earlier still. (Staged through shared memory with cp.async, the
+//    gathers cost 7.5 shared-memory wavefronts per copy and the data path of
+//    L1 was 67% busy; with plain loads it is 37%: 898 -> 851 us per force
+//    call at 1,000,002 atoms, 24.4 -> 23.5 at 11,997.)
+//  - Groups whose j atoms all sit at the center image skip the addition of
+//    S = 0 and its shared loads (851 -> 821 us at 1,000,002 atoms).
+//  - The row pairs' positions and charges and their LJ coefficients by j
+//    type sit in per-warp shared tables, already in packed order.
 //  - j forces stay in registers over the 4 rows and go out with one
 //    16-byte vector atomic per lane (fsort is float4 per slot).
 //  - i forces stay in registers over the whole half and are reduced across
@@ -32,10 +36,11 @@
 //    across halves in a per-warp shared pair (no registers held across
 //    halves), FP64 atomics per system when the warp moves to another
 //    system or finishes.
-//  - Every half comes from the work counter, the first too: taking each
-//    warp's first half from its grid index instead was 1 us slower at
-//    96,000 atoms (the counter spreads the largest halves over the SMs as
-//    they free up).
+//  - Halves are handed out in cluster order. Half lists make the first
+//    clusters' lists the longest and the last ones' the shortest, so the
+//    launch ends with short items as it would in sorted order, and neither
+//    an order array nor the sorting before it is needed (sorted: 1 us
+//    slower per call at 96,000 atoms, 4 us at 1,000,002).
 #include "nb_pair_x2.cuh"
 #include "nb_warp.cuh"
 
@@ -49,7 +54,6 @@ struct VtParams {
     const unsigned *vt_mask;  // 4 x 8 bits per tile
     const int *half_start;
     const int *half_len;
-    const int *order;         // i-clusters by decreasing list length, or NULL
     const float *ljparams;
     nb_dev_state *st;
     double *energies;         // [2 nsys]
@@ -76,13 +80,6 @@ __device__ __forceinline__ void flush_energies_vt(double *e, double *out) {
     e[1] = 0.0;
 }
 
-// Per-lane staging of one group of 32 gathered j atoms (4 tiles of 8).
-struct VtStage {
-    float4 xj[32];
-    int tj[32];
-    unsigned m[32];
-};
-
 // The lane's slot word of group g of the half with tiles [t0, t1): its j
 // atom's slot and shift, or the pad slot past the end (the load then reads
 // tile t0, so that no lane branches).
@@ -94,16 +91,23 @@ __device__ __forceinline__ int slot_word(const VtParams &p, int t0, int t1, int 
     return live ? w : (int)((unsigned)p.pad_slot | ((unsigned)NB_SHIFT_CENTER << 27));
 }
 
-// Issues the copies of group g (slot word v) into st: the tile's mask word
-// (zero-filled past the end), the j atom's coordinates and charge, its type.
-__device__ __forceinline__ void stage_copies(const VtParams &p, VtStage &st, int v, int t0, int t1, int g,
-                                             int lane) {
+// The lane's j atom of one group: coordinates and charge, type, mask word of
+// its tile (0 past the end).
+struct VtJ {
+    float4 x;
+    int t;
+    unsigned m;
+};
+
+__device__ __forceinline__ VtJ load_j(const VtParams &p, int v, int t0, int t1, int g, int lane) {
     const int tile = t0 + 4 * g + (lane >> 3);
-    const bool live = tile < t1;
-    cp_async4_zfill(&st.m[lane], p.vt_mask + (live ? tile : t0), live ? 4u : 0u);
     const int slot = v & 0x07ffffff;
-    cp_async16(&st.xj[lane], p.xq + slot);
-    cp_async4(&st.tj[lane], p.tsort + slot);
+    VtJ j;
+    j.m = 0u;
+    if (tile < t1) j.m = p.vt_mask[tile];
+    j.x = p.xq[slot];
+    j.t = p.tsort[slot];
+    return j;
 }
 
 // j-stationary kernel over gathered tiles. A warp takes one half i-cluster
@@ -112,22 +116,19 @@ __device__ __forceinline__ void stage_copies(const VtParams &p, VtStage &st, int
 // pairs of packed arithmetic. j forces stay in registers for the 4 pairs
 // and go out with one 16-byte vector atomic per lane (fsort is float4 per
 // slot); i forces stay in registers for the whole half and are reduced
-// across the warp at its end. Group g + 1 is copied (cp.async) into the
-// other buffer while group g is computed, and group g + 2's slot words load
-// meanwhile.
+// across the warp at its end. Group g + 1's j atoms load while group g is
+// computed, and group g + 2's slot words meanwhile.
 // Dynamic shared memory: the ntype x ntype LJ table, then per warp 3 float4
 // per j type (see s_lj2).
-// 640 / THREADS resident CTAs per SM (5 of 128 threads, the default shape)
-// leave up to 102 registers per thread (89 used, no spills): the 4 rows'
-// forces and the j atom's data stay in registers; the rows' positions,
-// charges and LJ coefficients are read from the per-warp shared tables.
-// 6 CTAs at 80 registers (and 3 of 256) were 3.5-4 us slower at 96,000
-// atoms, 4 CTAs at up to 128 registers 0.5 us slower.
+// Bound by the FMA pipe and instruction issue together, each about 61% busy
+// (a packed instruction holds the pipe for 2 cycles), with 5 warps per
+// scheduler to cover a half's chain of dependent loads. 640 / THREADS
+// resident CTAs per SM leave up to 96 registers per thread; 6 CTAs of 128
+// (80 registers) and 4 were slower.
 template <bool ENERGY, bool COUNT, int THREADS, int COUL>
 __global__ void __launch_bounds__(THREADS, 640 / THREADS) k_force_vt(VtParams p) {
     constexpr int kWarps = THREADS / 32;
     extern __shared__ float4 s_lj[];
-    __shared__ VtStage s_st[kWarps][2];
     __shared__ float4 s_shift[kWarps][27];  // the warp's copy of its system's shift vectors
     int shift_sys = -1;
     __shared__ float4 s_xi[kWarps][4];
@@ -176,7 +177,7 @@ __global__ void __launch_bounds__(THREADS, 640 / THREADS) k_force_vt(VtParams p)
         int ci = 0;
         if (w < n0) {
             hw = w;
-            ci = p.order ? p.order[hw >> 1] : (int)(hw >> 1);
+            ci = (int)(hw >> 1);
         } else if (w < nwork) {
             reg = 1u;
             hw = p.nl_list ? (unsigned)p.nl_list[w - n0] : w - n0;
@@ -198,7 +199,7 @@ __global__ void __launch_bounds__(THREADS, 640 / THREADS) k_force_vt(VtParams p)
         }
         const int ibase = ci * NB_CLUSTER + 4 * h;
         int v = slot_word(p, t0, t1, 0, lane);
-        stage_copies(p, s_st[warp][0], v, t0, t1, 0, lane);
+        VtJ j = load_j(p, v, t0, t1, 0, lane);
         int vnext = slot_word(p, t0, t1, 1, lane);
         if (lane < 4) {
             const float4 x = p.xq[ibase + lane];
@@ -210,7 +211,6 @@ __global__ void __launch_bounds__(THREADS, 640 / THREADS) k_force_vt(VtParams p)
         for (int k = 0; k < 2; ++k) fix[k] = fiy[k] = fiz[k] = make_float2(0.f, 0.f);
         float2 ec2 = make_float2(0.f, 0.f), elj2 = make_float2(0.f, 0.f);
         const int ngroups = (t1 - t0 + 3) >> 2;
-        cp_async_wait_all();
         __syncwarp();
         if (lane < 2) {
             const float4 a = s_xi[warp][2 * lane], b = s_xi[warp][2 * lane + 1];
@@ -222,30 +222,45 @@ __global__ void __launch_bounds__(THREADS, 640 / THREADS) k_force_vt(VtParams p)
             const float4 c2 = s_lj[s_tr[warp][2] + t], c3 = s_lj[s_tr[warp][3] + t];
             s_lj2[3 * t + 0] = make_float4(c0.x, c1.x, c0.y, c1.y);
             s_lj2[3 * t + 1] = make_float4(c2.x, c3.x, c2.y, c3.y);
-            s_lj2[3 * t + 2] = make_float4(-c0.z, -c1.z, -c2.z, -c3.z);
+            if (ENERGY) s_lj2[3 * t + 2] = make_float4(-c0.z, -c1.z, -c2.z, -c3.z);
         }
         __syncwarp();
         for (int g = 0; g < ngroups; ++g) {
-            VtStage &cs = s_st[warp][g & 1];
-            const float4 xj = cs.xj[lane];
-            const float4 S = s_shift[warp][(unsigned)v >> 27];
-            const int tj = cs.tj[lane];
-            const unsigned mrow = cs.m[lane] >> (lane & 7);  // bit 8a: row a
+            const float4 xj = j.x;
+            const int tj = j.t;
+            const unsigned mrow = j.m >> (lane & 7);  // bit 8a: row a
             const int slot = v & 0x07ffffff;
             const float2 nxjx = nb_f2(-xj.x), nxjy = nb_f2(-xj.y), nxjz = nb_f2(-xj.z), qj = nb_f2(xj.w);
-            const float2 Sx = nb_f2(S.x), Sy = nb_f2(S.y), Sz = nb_f2(S.z);
-            const float4 nsh = s_lj2[3 * tj + 2];
-            float2 gjx = make_float2(0.f, 0.f), gjy = gjx, gjz = gjx;
-            // the next group's copies overlap this whole group, and the slot word after it is
-            // loaded a group ahead (past the last group: pad copies)
-            stage_copies(p, s_st[warp][(g + 1) & 1], vnext, t0, t1, g + 1, lane);
-            const int vafter = slot_word(p, t0, t1, g + 2, lane);
+            // d = (y_a - y_b) + S; a group whose atoms all sit at the center image skips S = 0
+            float2 dx[2], dy[2], dz[2], qi[2];
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 const float4 xa = s_xp[warp][k][0], xb = s_xp[warp][k][1];
+                dx[k] = __fadd2_rn(make_float2(xa.x, xa.y), nxjx);
+                dy[k] = __fadd2_rn(make_float2(xa.z, xa.w), nxjy);
+                dz[k] = __fadd2_rn(make_float2(xb.x, xb.y), nxjz);
+                qi[k] = make_float2(xb.z, xb.w);
+            }
+            if (__any_sync(0xffffffffu, ((unsigned)v >> 27) != NB_SHIFT_CENTER)) {
+                const float4 S = s_shift[warp][(unsigned)v >> 27];
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    dx[k] = __fadd2_rn(dx[k], nb_f2(S.x));
+                    dy[k] = __fadd2_rn(dy[k], nb_f2(S.y));
+                    dz[k] = __fadd2_rn(dz[k], nb_f2(S.z));
+                }
+            }
+            float4 nsh = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (ENERGY) nsh = s_lj2[3 * tj + 2];
+            float2 gjx = make_float2(0.f, 0.f), gjy = gjx, gjz = gjx;
+            // the next group's j atoms load during this whole group, and the slot words after it
+            // a group ahead (past the last group: the pad slot)
+            j = load_j(p, vnext, t0, t1, g + 1, lane);
+            const int vafter = slot_word(p, t0, t1, g + 2, lane);
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
                 const int c2 = nb_pair_x2<ENERGY, COUL>(
-                    make_float2(xa.x, xa.y), make_float2(xa.z, xa.w), make_float2(xb.x, xb.y),
-                    make_float2(xb.z, xb.w), nxjx, nxjy, nxjz, qj, Sx, Sy, Sz, s_lj2[3 * tj + k],
+                    dx[k], dy[k], dz[k], qi[k], qj, s_lj2[3 * tj + k],
                     k == 0 ? make_float2(nsh.x, nsh.y) : make_float2(nsh.z, nsh.w), ((mrow >> (16 * k)) & 1u) != 0u,
                     ((mrow >> (16 * k + 8)) & 1u) != 0u, p.cc.rc2, p.cc2, fix[k], fiy[k], fiz[k], gjx, gjy, gjz, ec2,
                     elj2);
@@ -256,8 +271,6 @@ __global__ void __launch_bounds__(THREADS, 640 / THREADS) k_force_vt(VtParams p)
                           make_float4(-(gjx.x + gjx.y), -(gjy.x + gjy.y), -(gjz.x + gjz.y), 0.0f));
             v = vnext;
             vnext = vafter;
-            cp_async_wait_all();
-            __syncwarp();
         }
         // i forces: row a component c is value 4a + c; lanes 2k hold value k
         float r[16];
@@ -336,7 +349,6 @@ cudaError_t nb_launch_force_vt(nb_pairlist *pl, int ntype, const float *ljparams
     p.vt_mask = pl->vt_mask;
     p.half_start = pl->half_start;
     p.half_len = pl->half_len;
-    p.order = pl->sorted ? pl->ci_order : nullptr;
     p.ljparams = ljparams;
     p.st = pl->st;
     p.energies = energies;

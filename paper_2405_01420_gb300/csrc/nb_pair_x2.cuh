@@ -72,22 +72,16 @@ __device__ __forceinline__ float2 nb_erfcx_x2(float2 x) {
     return __fmul2_rn(p, y);
 }
 
-// Rows a, b (positions xi*, f q_i in qi) against j (negated position
-// nxj*, charge qj, all lanes equal) with shift S*. lj = (C6_a, C6_b,
-// C12_a, C12_b), nshlj = minus the LJ shifts of a and b. in_a, in_b: the
-// list mask bits. Adds the rows' forces to fi*, the j force (positive sign,
+// Rows a, b (displacements d* = (y_a - y_b) + S, f q_i in qi) against j
+// (charge qj, both lanes equal). lj = (C6_a, C6_b, C12_a, C12_b), nshlj =
+// minus the LJ shifts of a and b. in_a, in_b: the list mask bits. Adds the rows' forces to fi*, the j force (positive sign,
 // summed over rows) to gj*, and with ENERGY the pair energies to ec, elj.
 // Returns the number of the two pairs within rc.
 template <bool ENERGY, int COUL>
-__device__ __forceinline__ int nb_pair_x2(const float2 xix, const float2 xiy, const float2 xiz, const float2 qi,
-                                          const float2 nxjx, const float2 nxjy, const float2 nxjz, const float2 qj,
-                                          const float2 Sx, const float2 Sy, const float2 Sz, const float4 lj,
-                                          const float2 nshlj, const bool in_a, const bool in_b, const float rc2,
+__device__ __forceinline__ int nb_pair_x2(const float2 dx, const float2 dy, const float2 dz, const float2 qi,
+                                          const float2 qj, const float4 lj, const float2 nshlj, const bool in_a, const bool in_b, const float rc2,
                                           const nb_coul2 &cc, float2 &fix, float2 &fiy, float2 &fiz, float2 &gjx,
                                           float2 &gjy, float2 &gjz, float2 &ec, float2 &elj) {
-    const float2 dx = __fadd2_rn(__fadd2_rn(xix, nxjx), Sx);
-    const float2 dy = __fadd2_rn(__fadd2_rn(xiy, nxjy), Sy);
-    const float2 dz = __fadd2_rn(__fadd2_rn(xiz, nxjz), Sz);
     const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
     const bool ia = in_a && (r2.x < rc2);
     const bool ib = in_b && (r2.y < rc2);
