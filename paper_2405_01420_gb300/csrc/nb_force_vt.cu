@@ -42,6 +42,11 @@
 //    launch ends with short items as it would in sorted order, and neither
 //    an order array nor the sorting before it is needed (sorted: 1 us
 //    slower per call at 96,000 atoms, 4 us at 1,000,002).
+//  - First items (FIRST_BY_INDEX): from the work counter, or from the warp's index in
+//    the grid. The counter serves one warp per 1.3 ns, so 3,040 warps start
+//    over 4 us: a loss when each takes only a few halves (11,997 atoms: 22.0
+//    us per call from the counter, 18.1 from the index), a gain of 1 to 5%
+//    when it takes many (the warps' phases are spread from the start).
 #include "nb_pair_x2.cuh"
 #include "nb_warp.cuh"
 
@@ -111,6 +116,13 @@ __device__ __forceinline__ VtJ load_j(const VtParams &p, int v, int t0, int t1, 
     return j;
 }
 
+// The next work item: from the counter, past the items handed out by index.
+__device__ __forceinline__ unsigned take_item(const VtParams &p, unsigned by_index, int lane) {
+    unsigned w = 0;
+    if (lane == 0) w = atomicAdd(&p.st->work, 1u);
+    return __shfl_sync(0xffffffffu, w, 0) + by_index;
+}
+
 // j-stationary kernel over gathered tiles. A warp takes one half i-cluster
 // (4 i rows) at a time; its tiles are read in groups of 4 (32 j atoms, one
 // per lane), and each lane computes its j atom against the 4 rows, two row
@@ -123,11 +135,11 @@ __device__ __forceinline__ VtJ load_j(const VtParams &p, int v, int t0, int t1, 
 // per j type (see s_lj2).
 // Bound by the FMA pipe and instruction issue together, each about 61% busy
 // (a packed instruction holds the pipe for 2 cycles), with 5 warps per
-// scheduler to cover a half's chain of dependent loads. 640 / THREADS
-// resident CTAs per SM leave up to 96 registers per thread; 6 CTAs of 128
-// (80 registers) and 4 were slower.
-template <bool ENERGY, bool COUNT, int THREADS, int COUL>
-__global__ void __launch_bounds__(THREADS, 640 / THREADS) k_force_vt(VtParams p) {
+// scheduler to cover a half's chain of dependent loads. RES x THREADS
+// resident threads per SM set the register cap; pick_shape says which is
+// taken when.
+template <bool ENERGY, bool COUNT, int THREADS, int RES, bool FIRST_BY_INDEX, int COUL>
+__global__ void __launch_bounds__(THREADS, RES) k_force_vt(VtParams p) {
     constexpr int kWarps = THREADS / 32;
     extern __shared__ float4 s_lj[];
     __shared__ float4 s_shift[kWarps][27];  // the warp's copy of its system's shift vectors
@@ -171,10 +183,10 @@ __global__ void __launch_bounds__(THREADS, 640 / THREADS) k_force_vt(VtParams p)
     int cur_sys = -1;
     unsigned cnt = 0;
 
+    const unsigned by_index = FIRST_BY_INDEX ? gridDim.x * kWarps : 0u;
+    unsigned w = FIRST_BY_INDEX ? blockIdx.x * kWarps + warp : 0u;
+    if (!FIRST_BY_INDEX) w = take_item(p, 0u, lane);
     for (;;) {
-        unsigned w = 0;
-        if (lane == 0) w = atomicAdd(&p.st->work, 1u);
-        w = __shfl_sync(0xffffffffu, w, 0);
         unsigned reg = 0u, hw = 0u;
         int ci = 0;
         if (w < n0) {
@@ -194,7 +206,10 @@ __global__ void __launch_bounds__(THREADS, 640 / THREADS) k_force_vt(VtParams p)
         if (w >= nwork) break;
         const size_t hidx = (size_t)reg * p.reg_stride + 2 * ci + h;
         const int t0 = p.half_start[hidx], t1 = t0 + p.half_len[hidx];
-        if (t1 <= t0) continue;
+        if (t1 <= t0) {
+            w = take_item(p, by_index, lane);
+            continue;
+        }
         if (csys != shift_sys) {
             if (lane < 27) s_shift[warp][lane] = p.sys_shift[27 * csys + lane];
             shift_sys = csys;
@@ -306,6 +321,7 @@ __global__ void __launch_bounds__(THREADS, 640 / THREADS) k_force_vt(VtParams p)
             }
         }
         __syncwarp();
+        w = take_item(p, by_index, lane);
     }
     if (COUNT) {
         unsigned long long c64 = cnt;
@@ -315,23 +331,54 @@ __global__ void __launch_bounds__(THREADS, 640 / THREADS) k_force_vt(VtParams p)
 }
 
 using VtFn = void (*)(VtParams);
+
+// Launch shapes (threads, resident CTAs per SM, first items by index). The
+// default of 128 threads picks by the halves there are per warp of the grid;
+// microseconds per force call at 5 CTAs from the counter, then the shape
+// taken (rc 1.0, water):
+//   without energies, up to 3.5 halves per warp: 5 CTAs by index
+//     (6,000 atoms 21.1 -> 15.5, 24,000 26.7 -> 26.0, 36,000 34.5 -> 34.2;
+//     48,000 42.2 -> 42.5, 96,000 80.8 -> 81.5)
+//   without energies, from 10 halves per warp: 6 CTAs (77 registers)
+//     (96,000 80.8 -> 81.0, 192,000 155 -> 152, 1,000,002 740 -> 712)
+//   with energies, up to 6 halves per warp of 4 CTAs: 4 CTAs by index
+//     (6,000 25.4 -> 17.2, 24,000 36.1 -> 34.2, 48,000 57.4 -> 55.5;
+//     96,000 102.3 -> 106.8)
+// Counting kernels and 256 threads have one shape.
+enum { kShape256, kShapeCounter, kShapeIndex, kShapeMany, kShapes };
+
+int pick_shape(bool energy, bool count, int threads, long long halves, int num_sms) {
+    if (threads == 256) return kShape256;
+    if (count) return kShapeCounter;
+    const long long per_cta = 4LL * num_sms;  // warps of the grid per resident CTA
+    if (energy) return halves <= 6 * 4 * per_cta ? kShapeIndex : kShapeCounter;
+    if (2 * halves <= 7 * 5 * per_cta) return kShapeIndex;
+    return halves >= 10 * 5 * per_cta ? kShapeMany : kShapeCounter;
+}
+
 template <bool E, bool C, int K>
-VtFn pick_vt_shape(int threads) {
-    return threads == 128 ? k_force_vt<E, C, 128, K> : k_force_vt<E, C, 256, K>;
+VtFn pick_vt_shape(int shape) {
+    if (shape == kShape256) return k_force_vt<E, C, 256, 2, false, K>;
+    if constexpr (!C) {
+        if (shape == kShapeIndex) return k_force_vt<E, C, 128, E ? 4 : 5, true, K>;
+        if constexpr (!E)
+            if (shape == kShapeMany) return k_force_vt<E, C, 128, 6, false, K>;
+    }
+    return k_force_vt<E, C, 128, 5, false, K>;
 }
 
 template <bool E, bool C>
-VtFn pick_vt(int threads, int coul) {
-    if (coul == NB_COULK_RF) return pick_vt_shape<E, C, NB_COULK_RF>(threads);
-    if (coul == NB_COULK_EWALD_SHIFT) return pick_vt_shape<E, C, NB_COULK_EWALD_SHIFT>(threads);
-    return pick_vt_shape<E, C, NB_COULK_EWALD>(threads);
+VtFn pick_vt(int shape, int coul) {
+    if (coul == NB_COULK_RF) return pick_vt_shape<E, C, NB_COULK_RF>(shape);
+    if (E && coul == NB_COULK_EWALD_SHIFT) return pick_vt_shape<E, C, NB_COULK_EWALD_SHIFT>(shape);
+    return pick_vt_shape<E, C, NB_COULK_EWALD>(shape);  // the shift does not change forces
 }
 
 struct Occ {
     size_t smem;
     int per_sm;
 };
-Occ g_vt_occ[3][2][2][2] = {};
+Occ g_vt_occ[3][2][2][kShapes] = {};
 
 }  // namespace
 
@@ -367,10 +414,13 @@ cudaError_t nb_launch_force_vt(nb_pairlist *pl, int ntype, const float *ljparams
     const int e = energies ? 1 : 0;
     const int c = (pl->flags & NB_FLAG_COUNT_PAIRS) ? 1 : 0;
     const int threads = pl->force_threads == 256 ? 256 : 128;
-    VtFn fn = e ? (c ? pick_vt<true, true>(threads, coul) : pick_vt<true, false>(threads, coul))
-                : (c ? pick_vt<false, true>(threads, coul) : pick_vt<false, false>(threads, coul));
+    // halves of all systems: one cluster per 8 atoms and at most one more per column
+    const long long halves = 2LL * (pl->n_atoms / NB_CLUSTER + pl->ncol);
+    const int shape = pick_shape(e, c, threads, halves, pl->num_sms);
+    VtFn fn = e ? (c ? pick_vt<true, true>(shape, coul) : pick_vt<true, false>(shape, coul))
+                : (c ? pick_vt<false, true>(shape, coul) : pick_vt<false, false>(shape, coul));
     const size_t smem = sizeof(float4) * ((size_t)ntype * ntype + 3 * (size_t)ntype * (threads / 32));
-    Occ &occ = g_vt_occ[coul][e][c][threads == 128];
+    Occ &occ = g_vt_occ[coul][e][c][shape];
     if (occ.per_sm == 0 || occ.smem != smem) {  // resident CTAs for this LJ table size
         int n = 0;
         cudaError_t err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, (const void *)fn, threads, smem);
