@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(THREADS, RES) k_force_vt(VtParams p) {
     for (int k = threadIdx.x; k < nt2; k += blockDim.x) {
         const float c6 = p.ljparams[2 * k], c12 = p.ljparams[2 * k + 1];
         s_lj[k] = ENERGY ? make_float4(c6, c12, c12 * p.rc12inv - c6 * p.rc6inv, 0.0f)
-                         : make_float4(-6.0f * c6, 12.0f * c12, 0.0f, 0.0f);
+                         : make_float4(-6.0f * c6, nb_lj12_scale(COUL) * c12, 0.0f, 0.0f);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const unsigned ds = p.st->cur_d2_search, dp = p.st->cur_d2_prune;

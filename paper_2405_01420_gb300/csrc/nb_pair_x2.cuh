@@ -114,10 +114,14 @@ __device__ __forceinline__ float2 nb_ewald_force_x2(const nb_coul2 &cc, const fl
     return __fmul2_rn(__fmul2_rn(p, y), __fmul2_rn(ex, rinv));
 }
 
+// Scale of C12 in the force-only LJ table: the reaction field's pair force
+// takes 12 C12, Ewald's C12 as it is.
+__host__ __device__ constexpr float nb_lj12_scale(int coul) { return coul == NB_COULK_RF ? 12.0f : 1.0f; }
+
 // Rows a, b (displacements d* = (y_a - y_b) + S, f q_i in qi) against j
 // (charge qj, both lanes equal). lj = (C6_a, C6_b, C12_a, C12_b), or without
-// ENERGY (-6 C6_a, -6 C6_b, 12 C12_a, 12 C12_b); nshlj = minus the LJ shifts
-// of a and b. in_a, in_b: the list mask bits. Adds the rows' forces to fi*, the j force (positive sign,
+// ENERGY (-6 C6_a, -6 C6_b, k C12_a, k C12_b) with k = nb_lj12_scale(COUL);
+// nshlj = minus the LJ shifts of a and b. in_a, in_b: the list mask bits. Adds the rows' forces to fi*, the j force (positive sign,
 // summed over rows) to gj*, and with ENERGY the pair energies to ec, elj.
 // Returns the number of the two pairs within rc.
 template <bool ENERGY, int COUL>
@@ -148,14 +152,19 @@ __device__ __forceinline__ int nb_pair_x2(const float2 dx, const float2 dy, cons
             s = __ffma2_rn(__fmul2_rn(qq, __ffma2_rn(cc.c2b, ex, a)), rinv2, slj);
         }
     } else {
-        // no energies, so no v6 and v12 of their own: 12 C12/r^6 - 6 C6 in one FMA
-        const float2 w = __ffma2_rn(make_float2(lj.z, lj.w), rinv6, make_float2(lj.x, lj.y));
         if (COUL == NB_COULK_RF) {
+            // no energies, so no v6 and v12 of their own: 12 C12/r^6 - 6 C6 in one FMA
+            const float2 w = __ffma2_rn(make_float2(lj.z, lj.w), rinv6, make_float2(lj.x, lj.y));
             s = __ffma2_rn(qq, __ffma2_rn(rinv, rinv2, cc.m2krf), __fmul2_rn(w, __fmul2_rn(rinv6, rinv2)));
         } else {
+            // the repulsion is rounded as with energies: what is derived from the forces of close
+            // pairs (the gradient of a force-matching loss) is the same with and without them
+            const float2 v12n = __fmul2_rn(__fmul2_rn(make_float2(lj.z, lj.w), rinv6), rinv6);
+            const float2 slj = __fmul2_rn(
+                __ffma2_rn(nb_f2(12.0f), v12n, __fmul2_rn(make_float2(lj.x, lj.y), rinv6)), rinv2);
             float2 ex;
             const float2 e = nb_ewald_force_x2(cc, r2, rinv, ex);
-            s = __fmul2_rn(__ffma2_rn(w, rinv6, __fmul2_rn(qq, e)), rinv2);
+            s = __ffma2_rn(__fmul2_rn(qq, e), rinv2, slj);
         }
     }
     s.x = ia ? s.x : 0.0f;
