@@ -9,14 +9,17 @@
 //  - i side: registers over the whole half, reduced across the warp at its
 //    end (reduce-scatter), one vector atomic per row.
 //  - dL/dC6, dL/dC12: per-lane FP32 accumulators for each (row, j type),
-//    kept in shared memory (one column per lane, so a lane's adds never
-//    meet another lane's bank), reduced across the warp once per half by a
-//    skewed read (lane k sums row k, starting at bank k) and added in FP64
-//    to the unsymmetrised [ntype][ntype][2] accumulator. In registers they
-//    took 32 of them and held the kernel at 4 warps per scheduler.
+//    kept in shared memory, a row pair's four in one float4 of the lane's
+//    own column (any 8 lanes cover the 32 banks whatever their types),
+//    reduced across the warp once per half by a skewed read (lane k sums
+//    value k, starting at column k) and added in FP64 to the unsymmetrised
+//    [ntype][ntype][2] accumulator. In registers they took 32 of them and
+//    held the kernel at 4 warps per scheduler.
 // Group g + 1's j data (coordinates and charge, g, type, mask word) are
-// copied into shared memory with cp.async from the start of group g, their
-// slot words loaded one group earlier still.
+// loaded into registers while group g is computed, their slot words one
+// group earlier still; groups at the center image skip S = 0; halves are
+// taken in cluster order (nb_force_vt.cu gives the reasons, which are the
+// same here).
 #include "nb_pair_x2.cuh"
 #include "nb_warp.cuh"
 
@@ -24,7 +27,9 @@ namespace {
 
 constexpr int kBvtThreads = 128;
 constexpr int kBvtWarps = kBvtThreads / 32;
-constexpr int kBvtCtasPerSm = 4;  // up to 128 registers (115 used); 5 CTAs at 102 were 1.3 us slower at 24k atoms, 6 at 80 slower still
+// 4 CTAs: up to 128 registers (123 used, no spills). The adjoint pass at 24,000 atoms: 101.5 us with the
+// j data staged by cp.async, a Horner erfcx and scalar LJ accumulators, 98.8 us as it is now.
+constexpr int kBvtCtasPerSm = 4;
 
 struct BvtParams {
     const float4 *xq;
@@ -36,7 +41,6 @@ struct BvtParams {
     const unsigned *vt_mask;  // 4 x 8 bits per tile
     const int *half_start;
     const int *half_len;
-    const int *order;         // i-clusters by decreasing work, or NULL
     const float *ljparams;
     nb_dev_state *st;
     const float4 *sys_shift;  // [27 nsys]
@@ -51,13 +55,6 @@ struct BvtParams {
     int reg_stride;  // 2 nc_max
 };
 
-struct BvtStage {
-    float4 xj[32];
-    float4 gj[32];
-    int tj[32];
-    unsigned m[32];
-};
-
 // The lane's slot word of group g of the half with tiles [t0, t1): its j
 // atom's slot and shift, or the pad slot past the end (the load then reads
 // tile t0, so that no lane branches).
@@ -69,26 +66,34 @@ __device__ __forceinline__ int slot_word_adj(const BvtParams &p, int t0, int t1,
     return live ? w : (int)((unsigned)p.pad_slot | ((unsigned)NB_SHIFT_CENTER << 27));
 }
 
-// Issues the copies of group g (slot word v) into st: the tile's mask word
-// (zero-filled past the end), the j atom's coordinates and charge, g, type.
-__device__ __forceinline__ void stage_adj(const BvtParams &p, BvtStage &st, int v, int t0, int t1, int g, int lane) {
+// The lane's j atom of one group: coordinates and charge, g, type, mask word
+// of its tile (0 past the end).
+struct BvtJ {
+    float4 x, g;
+    int t;
+    unsigned m;
+};
+
+__device__ __forceinline__ BvtJ load_adj(const BvtParams &p, int v, int t0, int t1, int g, int lane) {
     const int tile = t0 + 4 * g + (lane >> 3);
-    const bool live = tile < t1;
-    cp_async4_zfill(&st.m[lane], p.vt_mask + (live ? tile : t0), live ? 4u : 0u);
     const int slot = v & 0x07ffffff;
-    cp_async16(&st.xj[lane], p.xq + slot);
-    cp_async16(&st.gj[lane], p.gsort + slot);
-    cp_async4(&st.tj[lane], p.tsort + slot);
+    BvtJ j;
+    j.m = 0u;
+    if (tile < t1) j.m = p.vt_mask[tile];
+    j.x = p.xq[slot];
+    j.g = p.gsort[slot];
+    j.t = p.tsort[slot];
+    return j;
 }
 
 template <int NT, int COUL>
 __global__ void __launch_bounds__(kBvtThreads, kBvtCtasPerSm) k_backward_vt(BvtParams p) {
-    constexpr int kAcc = 4 * NT * 2;  // (row a, j type t, C6 / C12) accumulators per lane
+    constexpr int kAcc = 4 * NT * 2;  // (row a, j type t, C6 / C12) accumulators per lane: value (a NT + t) 2 + c
     // dynamic: the ntype x ntype LJ table (C6, C12, 0, 0), then per warp, by j type t, the half's
     // row pairs' (C6_a, C6_b, C12_a, C12_b) at [2t + k]
     extern __shared__ float4 s_lj[];
-    __shared__ BvtStage s_st[kBvtWarps][2];
-    __shared__ float s_acc[kBvtWarps][kAcc][32];  // [value][lane]
+    // per warp, row pair k, j type and lane: (C6 of row 2k, C12 of row 2k, C6 of row 2k + 1, C12 of row 2k + 1)
+    __shared__ float4 s_acc[kBvtWarps][2 * NT][32];
     __shared__ float4 s_shift[kBvtWarps][27];
     __shared__ float4 s_xi[kBvtWarps][4];  // (x, y, z, f q)
     __shared__ float4 s_gi[kBvtWarps][4];
@@ -114,9 +119,9 @@ __global__ void __launch_bounds__(kBvtThreads, kBvtCtasPerSm) k_backward_vt(BvtP
     const unsigned nhalf = 2u * (unsigned)p.st->nc;
     const unsigned nwork = nhalf * (unsigned)p.nreg;
     int shift_sys = -1;
-    float(*acc)[32] = s_acc[warp];
+    float4(*acc)[32] = s_acc[warp];
 #pragma unroll
-    for (int k = 0; k < kAcc; ++k) acc[k][lane] = 0.0f;
+    for (int k = 0; k < 2 * NT; ++k) acc[k][lane] = make_float4(0.f, 0.f, 0.f, 0.f);
 
     const unsigned nwarps = gridDim.x * kBvtWarps;
     for (unsigned it = 0;; ++it) {
@@ -129,7 +134,7 @@ __global__ void __launch_bounds__(kBvtThreads, kBvtCtasPerSm) k_backward_vt(BvtP
         }
         if (w >= nwork) break;
         const unsigned reg = w / nhalf, hw = w - reg * nhalf;
-        const int ci = p.order ? p.order[hw >> 1] : (int)(hw >> 1);
+        const int ci = (int)(hw >> 1);
         const int h = (int)(hw & 1u);
         const size_t hidx = (size_t)reg * p.reg_stride + 2 * ci + h;
         const int t0 = p.half_start[hidx], t1 = t0 + p.half_len[hidx];
@@ -141,7 +146,7 @@ __global__ void __launch_bounds__(kBvtThreads, kBvtCtasPerSm) k_backward_vt(BvtP
         }
         const int ibase = ci * NB_CLUSTER + 4 * h;
         int v = slot_word_adj(p, t0, t1, 0, lane);
-        stage_adj(p, s_st[warp][0], v, t0, t1, 0, lane);
+        BvtJ j = load_adj(p, v, t0, t1, 0, lane);
         int vnext = slot_word_adj(p, t0, t1, 1, lane);
         if (lane < 4) {
             const float4 x = p.xq[ibase + lane];
@@ -154,7 +159,6 @@ __global__ void __launch_bounds__(kBvtThreads, kBvtCtasPerSm) k_backward_vt(BvtP
 #pragma unroll
         for (int k = 0; k < 2; ++k) bix[k] = biy[k] = biz[k] = biq[k] = make_float2(0.f, 0.f);
         const int ngroups = (t1 - t0 + 3) >> 2;
-        cp_async_wait_all();
         __syncwarp();
         if (lane < 2) {
             const float4 a = s_xi[warp][2 * lane], b = s_xi[warp][2 * lane + 1];
@@ -174,47 +178,59 @@ __global__ void __launch_bounds__(kBvtThreads, kBvtCtasPerSm) k_backward_vt(BvtP
         __syncwarp();
         const float2 nk2 = nb_f2(-p.k2);
         for (int g = 0; g < ngroups; ++g) {
-            const BvtStage &cs = s_st[warp][g & 1];
-            const float4 xj = cs.xj[lane];
-            const float4 gj = cs.gj[lane];
-            const int tj = cs.tj[lane];
-            const unsigned mrow = cs.m[lane] >> (lane & 7);  // bit 8a: row a
-            const float4 S = s_shift[warp][(unsigned)v >> 27];
+            const int tj = j.t;
+            const unsigned mrow = j.m >> (lane & 7);  // bit 8a: row a
             const int slot = v & 0x07ffffff;
-            const float2 nxjx = nb_f2(-xj.x), nxjy = nb_f2(-xj.y), nxjz = nb_f2(-xj.z);
-            const float2 ngjx = nb_f2(-gj.x), ngjy = nb_f2(-gj.y), ngjz = nb_f2(-gj.z);
-            const float2 qj = nb_f2(xj.w), qj_f = nb_f2(xj.w * NB_COULOMB_F);
-            const float2 Sx = nb_f2(S.x), Sy = nb_f2(S.y), Sz = nb_f2(S.z);
-            float2 vjx = make_float2(0.f, 0.f), vjy = vjx, vjz = vjx, bjq = vjx;
-            // the next group's copies overlap this whole group, and the slot word after it is
-            // loaded a group ahead (past the last group: pad copies)
-            stage_adj(p, s_st[warp][(g + 1) & 1], vnext, t0, t1, g + 1, lane);
-            const int vafter = slot_word_adj(p, t0, t1, g + 2, lane);
+            const float2 nxjx = nb_f2(-j.x.x), nxjy = nb_f2(-j.x.y), nxjz = nb_f2(-j.x.z);
+            const float2 ngjx = nb_f2(-j.g.x), ngjy = nb_f2(-j.g.y), ngjz = nb_f2(-j.g.z);
+            const float2 qj = nb_f2(j.x.w), qj_f = nb_f2(j.x.w * NB_COULOMB_F);
+            // d = (y_a - y_b) + S; a group whose atoms all sit at the center image skips S = 0
+            float2 dx[2], dy[2], dz[2], qi_f[2];
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 const float4 xa = s_xp[warp][k][0], xb = s_xp[warp][k][1];
+                dx[k] = __fadd2_rn(make_float2(xa.x, xa.y), nxjx);
+                dy[k] = __fadd2_rn(make_float2(xa.z, xa.w), nxjy);
+                dz[k] = __fadd2_rn(make_float2(xb.x, xb.y), nxjz);
+                qi_f[k] = make_float2(xb.z, xb.w);
+            }
+            if (__any_sync(0xffffffffu, ((unsigned)v >> 27) != NB_SHIFT_CENTER)) {
+                const float4 S = s_shift[warp][(unsigned)v >> 27];
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    dx[k] = __fadd2_rn(dx[k], nb_f2(S.x));
+                    dy[k] = __fadd2_rn(dy[k], nb_f2(S.y));
+                    dz[k] = __fadd2_rn(dz[k], nb_f2(S.z));
+                }
+            }
+            float2 vjx = make_float2(0.f, 0.f), vjy = vjx, vjz = vjx, bjq = vjx;
+            // the next group's j atoms load during this whole group, and the slot words after it
+            // a group ahead (past the last group: the pad slot)
+            j = load_adj(p, vnext, t0, t1, g + 1, lane);
+            const int vafter = slot_word_adj(p, t0, t1, g + 2, lane);
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
                 const float4 ga = s_gp[warp][k][0], gb = s_gp[warp][k][1];
                 const float4 lj = s_ljp[2 * tj + k];
                 float2 d6, d12;
-                nb_pair_adj_x2<COUL>(make_float2(xa.x, xa.y), make_float2(xa.z, xa.w), make_float2(xb.x, xb.y),
-                                     make_float2(xb.z, xb.w), make_float2(ga.x, ga.y), make_float2(ga.z, ga.w),
-                                     make_float2(gb.x, gb.y), nxjx, nxjy, nxjz, qj, qj_f, ngjx, ngjy, ngjz, Sx, Sy, Sz,
-                                     make_float2(lj.x, lj.y), make_float2(lj.z, lj.w),
-                                     ((mrow >> (16 * k)) & 1u) != 0u, ((mrow >> (16 * k + 8)) & 1u) != 0u, p.cc.rc2,
-                                     p.cc2, nk2, bix[k], biy[k], biz[k], biq[k], vjx, vjy, vjz, bjq, d6, d12);
-                // the lane's own columns: tj < ntype <= NT (the gather keeps types in range)
-                acc[((2 * k) * NT + tj) * 2 + 0][lane] += d6.x;
-                acc[((2 * k) * NT + tj) * 2 + 1][lane] += d12.x;
-                acc[((2 * k + 1) * NT + tj) * 2 + 0][lane] += d6.y;
-                acc[((2 * k + 1) * NT + tj) * 2 + 1][lane] += d12.y;
+                nb_pair_adj_x2<COUL>(dx[k], dy[k], dz[k], qi_f[k], make_float2(ga.x, ga.y), make_float2(ga.z, ga.w),
+                                     make_float2(gb.x, gb.y), qj, qj_f, ngjx, ngjy, ngjz, make_float2(lj.x, lj.y),
+                                     make_float2(lj.z, lj.w), ((mrow >> (16 * k)) & 1u) != 0u,
+                                     ((mrow >> (16 * k + 8)) & 1u) != 0u, p.cc.rc2, p.cc2, nk2, bix[k], biy[k], biz[k],
+                                     biq[k], vjx, vjy, vjz, bjq, d6, d12);
+                // the lane's own column: tj < ntype <= NT (the gather keeps types in range)
+                float4 c = acc[k * NT + tj][lane];
+                c.x += d6.x;
+                c.y += d12.x;
+                c.z += d6.y;
+                c.w += d12.y;
+                acc[k * NT + tj][lane] = c;
             }
             if (slot != p.pad_slot)  // all padding lanes share one slot: no atomics there
                 atomicAdd(p.bsort + slot, make_float4(-(vjx.x + vjx.y), -(vjy.x + vjy.y), -(vjz.x + vjz.y),
                                                       bjq.x + bjq.y));
             v = vnext;
             vnext = vafter;
-            cp_async_wait_all();
-            __syncwarp();
         }
         // i side: value 4a + c (c = x, y, z, q); lane 8a then holds row a's x
         // and finds y, z, q 2, 4 and 6 lanes up
@@ -237,21 +253,20 @@ __global__ void __launch_bounds__(kBvtThreads, kBvtCtasPerSm) k_backward_vt(BvtP
             const float rq = __shfl_down_sync(0xffffffffu, r[0], 6);
             if ((lane & 7) == 0) atomicAdd(p.bsort + ibase + (lane >> 3), make_float4(r[0], ry, rz, rq));
         }
-        // LJ gradients: value k = (a NT + t) 2 + c, summed over the 32 lane columns by lane k,
-        // which starts at column k so that the 32 lanes read 32 different banks; each value is
-        // cleared as it is read
+        // LJ gradients: value k = (a NT + t) 2 + c, summed over the 32 columns by lane k, which starts
+        // at column k (4 lanes meet in the banks of a column, two of them in the same word)
         __syncwarp();
         if (lane < kAcc) {
+            const int a = lane / (2 * NT), t = (lane >> 1) % NT, c = lane & 1;
+            const float *val = reinterpret_cast<const float *>(acc[(a >> 1) * NT + t]) + 2 * (a & 1) + c;
             float sum = 0.0f;
 #pragma unroll 8
-            for (int i = 0; i < 32; ++i) {
-                const int col = (i + lane) & 31;
-                sum += acc[lane][col];
-                acc[lane][col] = 0.0f;
-            }
-            const int a = lane / (2 * NT), t = (lane >> 1) % NT, c = lane & 1;
+            for (int i = 0; i < 32; ++i) sum += val[4 * ((i + lane) & 31)];
             if (t < p.ntype && sum != 0.0f) atomicAdd(&p.glj_acc[2 * (s_tr[warp][a] + t) + c], (double)sum);
         }
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 2 * NT; ++k) acc[k][lane] = make_float4(0.f, 0.f, 0.f, 0.f);
         __syncwarp();
     }
 }
@@ -284,7 +299,6 @@ cudaError_t nb_launch_backward_vt(nb_pairlist *pl, int ntype, const float *ljpar
     p.vt_mask = pl->vt_mask;
     p.half_start = pl->half_start;
     p.half_len = pl->half_len;
-    p.order = pl->sorted ? pl->ci_order : nullptr;
     p.ljparams = ljparams;
     p.st = pl->st;
     p.sys_shift = pl->sys_shift;

@@ -198,27 +198,23 @@ __device__ __forceinline__ int nb_pair_x2(const float2 dx, const float2 dy, cons
 
 // Rows a, b (.x, .y) of the adjoint pair nb_pair_adj<true, COUL> against
 // one j atom, on the packed instructions: each lane performs the scalar
-// form's operations in its order (negations exact), so a row's values are
-// bit-equal to nb_pair_adj's. Inputs: the rows' positions xi*, f q_i in
-// qi_f and g in gi*; the j atom's negated position nxj*, charge qj, f q_j
-// in qj_f and negated g in ngj*; the shift S*; the rows' C6, C12 against
-// the j atom's type; the list mask bits in_a, in_b. Adds to the rows'
+// form's operations in its order (negations exact), but for the Ewald terms,
+// which come from nb_ewald_force_x2 (the adjoint has no energies), so the
+// LJ gradients of a row are bit-equal to nb_pair_adj's. Inputs: the rows'
+// displacements d* = (y_a - y_b) + S, f q_i in qi_f and g in gi*; the j
+// atom's charge qj, f q_j in qj_f and negated g in ngj*; the rows' C6, C12
+// against the j atom's type; the list mask bits in_a, in_b. Adds to the rows'
 // (dL/dx, dL/dq) in bi*; adds to vj* the vector v that the j atom's dL/dx
 // loses (subtract it once per j atom), and to bjq the j atom's dL/dq; d6,
 // d12 receive the two pairs' dL/dC6, dL/dC12 (0 when a pair does not count).
 template <int COUL>
-__device__ __forceinline__ void nb_pair_adj_x2(const float2 xix, const float2 xiy, const float2 xiz, const float2 qi_f,
-                                               const float2 gix, const float2 giy, const float2 giz,
-                                               const float2 nxjx, const float2 nxjy, const float2 nxjz,
-                                               const float2 qj, const float2 qj_f, const float2 ngjx,
-                                               const float2 ngjy, const float2 ngjz, const float2 Sx, const float2 Sy,
-                                               const float2 Sz, const float2 c6, const float2 c12, const bool in_a,
+__device__ __forceinline__ void nb_pair_adj_x2(const float2 dx, const float2 dy, const float2 dz, const float2 qi_f,
+                                               const float2 gix, const float2 giy, const float2 giz, const float2 qj,
+                                               const float2 qj_f, const float2 ngjx, const float2 ngjy,
+                                               const float2 ngjz, const float2 c6, const float2 c12, const bool in_a,
                                                const bool in_b, const float rc2, const nb_coul2 &cc, const float2 nk2,
                                                float2 &bix, float2 &biy, float2 &biz, float2 &biq, float2 &vjx,
                                                float2 &vjy, float2 &vjz, float2 &bjq, float2 &d6, float2 &d12) {
-    const float2 dx = __fadd2_rn(__fadd2_rn(xix, nxjx), Sx);
-    const float2 dy = __fadd2_rn(__fadd2_rn(xiy, nxjy), Sy);
-    const float2 dz = __fadd2_rn(__fadd2_rn(xiz, nxjz), Sz);
     const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
     const bool ia = in_a && (r2.x < rc2);
     const bool ib = in_b && (r2.y < rc2);
@@ -237,10 +233,8 @@ __device__ __forceinline__ void nb_pair_adj_x2(const float2 xix, const float2 xi
         Bc = __fadd2_rn(rinv3, cc.m2krf);  // 1/r^3 - 2 k_rf
         cpr = __fmul2_rn(__fmul2_rn(nb_f2(-3.0f), qq), rinv3);
     } else {
-        const float2 r = __fmul2_rn(r2, rinv);
-        const float2 ex = nb_exp2_x2(__fmul2_rn(cc.kexp, r2));
-        const float2 a = __fmul2_rn(__fmul2_rn(ex, nb_erfcx_x2(__fmul2_rn(cc.beta, r))), rinv);
-        Bc = __fmul2_rn(__ffma2_rn(cc.c2b, ex, a), rinv2);
+        float2 ex;
+        Bc = __fmul2_rn(nb_ewald_force_x2(cc, r2, rinv, ex), rinv2);
         cpr = __ffma2_rn(nb_f2(-3.0f), __fmul2_rn(qq, Bc), __fmul2_rn(__fmul2_rn(nk2, qq), ex));
     }
     const float2 s = __fadd2_rn(__fmul2_rn(qq, Bc), slj);
