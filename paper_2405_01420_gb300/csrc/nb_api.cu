@@ -462,9 +462,9 @@ extern "C" int nb_backward(nb_pairlist *pl, const float *coords, const float *q,
     DeviceGuard gd(pl->device);
     cudaStream_t s = (cudaStream_t)stream;
     NB_CUDA(sort_if_pending(pl, s));
-    NB_CUDA(nb_launch_gather(pl, coords, q, type, ntype, 0, nullptr, NB_PART_ALL, s));
-    NB_CUDA(nb_launch_backward(pl, ntype, ljparams, rc, beta, g, grad_x, grad_q, grad_lj,
-                               stale_bound2(pl->rlist, rc), stale_bound2(pl->r_inner, rc), s));
+    NB_CUDA(nb_launch_gather_adj(pl, coords, q, type, ntype, g, s));
+    NB_CUDA(nb_launch_backward(pl, ntype, ljparams, rc, beta, grad_x, grad_q, grad_lj, stale_bound2(pl->rlist, rc),
+                               stale_bound2(pl->r_inner, rc), s));
     return ok();
 }
 

@@ -12,16 +12,17 @@
 // The LJ gradient is reported for the symmetric matrix: each type pair's
 // derivative is split evenly between (ti, tj) and (tj, ti).
 //
-// k_gather_g   g (original order) -> gsort (cluster order); zeroes the
-//              gradient accumulators.
+// k_gather<true>  (nb_force.cu) the force call's gather, and g (original
+//              order) -> gsort (cluster order); zeroes the gradient
+//              accumulators.
 // k_backward   (8 x 8 cluster tiles; after a prune the gathered-tile form in
 //              nb_backward_vt.cu runs instead)
 //              one warp per i-cluster (work counter), list entries and their
 //              j data staged in shared memory, lane layout as in k_force;
 //              j-side gradients (x, y, z, q) reduce-scatter so every lane adds
 //              one component; per-lane LJ accumulators by j type (NT <= 4).
-// k_bwd_final  symmetrises the FP64 LJ accumulators into the output.
-// k_bwd_scatter  cluster order -> original order.
+// k_bwd_scatter  cluster order -> original order; its first block also
+//              symmetrises the FP64 LJ accumulators into the output.
 #include "nb_pair.cuh"
 
 namespace {
@@ -50,22 +51,6 @@ struct BwdParams {
     float stale_search2, stale_prune2;
     int has_inner;
 };
-
-__global__ void k_gather_g(int nmax_slots, const int *__restrict__ perm, const float *__restrict__ g,
-                           float4 *__restrict__ gsort, float4 *__restrict__ bsort, double *__restrict__ glj_acc,
-                           int nlj, const nb_dev_state *st) {
-    nb_pdl_wait();
-    nb_pdl_release();
-    const int nslot = min(st->nc * NB_CLUSTER, nmax_slots);
-    for (int slot = blockIdx.x * blockDim.x + threadIdx.x; slot < nslot; slot += gridDim.x * blockDim.x) {
-        const int atom = perm[slot];
-        gsort[slot] = atom < 0 ? make_float4(0.f, 0.f, 0.f, 0.f)
-                               : make_float4(g[3 * atom], g[3 * atom + 1], g[3 * atom + 2], 0.f);
-        bsort[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    if (blockIdx.x == 0)
-        for (int k = threadIdx.x; k < nlj; k += blockDim.x) glj_acc[k] = 0.0;
-}
 
 template <int NT>
 __device__ __forceinline__ void add_onehot(float (&acc)[NT][2], const int tj, const float d6, const float d12) {
@@ -218,21 +203,16 @@ __global__ void __launch_bounds__(kBwdThreads) k_backward(BwdParams p) {
     }
 }
 
-__global__ void k_bwd_final(int ntype, const double *__restrict__ acc, double *__restrict__ out) {
-    nb_pdl_wait();
-    nb_pdl_release();
-    const int k = threadIdx.x;
-    if (k >= ntype * ntype) return;
-    const int a = k / ntype, c = k % ntype;
-    const int kt = c * ntype + a;
-    out[2 * k] = 0.5 * (acc[2 * k] + acc[2 * kt]);
-    out[2 * k + 1] = 0.5 * (acc[2 * k + 1] + acc[2 * kt + 1]);
-}
-
 __global__ void k_bwd_scatter(int n, const int *__restrict__ pos, const float4 *__restrict__ bsort,
-                              float *__restrict__ grad_x, float *__restrict__ grad_q) {
+                              float *__restrict__ grad_x, float *__restrict__ grad_q, int ntype,
+                              const double *__restrict__ acc, double *__restrict__ grad_lj) {
     nb_pdl_wait();
     nb_pdl_release();
+    if (blockIdx.x == 0 && threadIdx.x < ntype * ntype) {
+        const int k = threadIdx.x, kt = (k % ntype) * ntype + k / ntype;
+        grad_lj[2 * k] = 0.5 * (acc[2 * k] + acc[2 * kt]);
+        grad_lj[2 * k + 1] = 0.5 * (acc[2 * k + 1] + acc[2 * kt + 1]);
+    }
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float4 v = bsort[pos[i]];
@@ -268,14 +248,9 @@ cudaError_t launch_bwd_nt(nb_pairlist *pl, const BwdParams &p, cudaStream_t s) {
 }  // namespace
 
 cudaError_t nb_launch_backward(nb_pairlist *pl, int ntype, const float *ljparams, float rc, float beta,
-                               const float *g, float *grad_x, float *grad_q, double *grad_lj,
-                               float stale_search2, float stale_prune2, cudaStream_t s) {
-    const int nslot = pl->nc_max * NB_CLUSTER;
-    const int nlj = 2 * ntype * ntype;
-    int gb = min((nslot + 255) / 256, pl->num_sms * 8);
-    cudaError_t e = nb_launch_pdl(k_gather_g, max(gb, 1), 256, 0, s, nslot, (const int *)pl->perm, g, pl->gsort,
-                                  pl->bsort, pl->glj_acc, nlj, (const nb_dev_state *)pl->st);
-    if (e != cudaSuccess) return e;
+                               float *grad_x, float *grad_q, double *grad_lj, float stale_search2,
+                               float stale_prune2, cudaStream_t s) {
+    cudaError_t e;
     BwdParams p;
     p.xq = pl->xq;
     p.tsort = pl->tsort;
@@ -307,9 +282,7 @@ cudaError_t nb_launch_backward(nb_pairlist *pl, int ntype, const float *ljparams
         e = nb_launch_excl_corr_adj(pl, rc, beta, s);
         if (e != cudaSuccess) return e;
     }
-    e = nb_launch_pdl(k_bwd_final, 1, 32, 0, s, ntype, (const double *)pl->glj_acc, grad_lj);
-    if (e != cudaSuccess) return e;
     const int n = pl->n_atoms;
     return nb_launch_pdl(k_bwd_scatter, (n + 255) / 256, 256, 0, s, n, (const int *)pl->pos, (const float4 *)pl->bsort,
-                         grad_x, grad_q);
+                         grad_x, grad_q, ntype, (const double *)pl->glj_acc, grad_lj);
 }

@@ -45,6 +45,12 @@ struct GatherParams {
     int ntype;
     int part;    // NB_PART_ALL / NB_PART_LOCAL (home atoms) / NB_PART_NONLOCAL (halo atoms)
     int n_home;  // atoms [0, n_home) are home atoms
+    // the adjoint's gather only
+    const float *g;   // dL/dF, original order
+    float4 *gsort;    // the same in cluster order
+    float4 *bsort;    // adjoint accumulators
+    double *glj_acc;  // adjoint LJ accumulators
+    int nlj;
 };
 
 __device__ __forceinline__ float warp_max(float v) {
@@ -52,6 +58,10 @@ __device__ __forceinline__ float warp_max(float v) {
     return v;
 }
 
+// ADJ: the gather of an adjoint call, which also brings dL/dF into cluster
+// order and clears the adjoint's accumulators in place of the forces'. One
+// kernel for both: a second one would read perm again and cost a launch.
+template <bool ADJ>
 __global__ void __launch_bounds__(256) k_gather(GatherParams p) {
     nb_pdl_wait();
     nb_pdl_release();
@@ -59,7 +69,13 @@ __global__ void __launch_bounds__(256) k_gather(GatherParams p) {
     float d2s_max = 0.0f, d2p_max = 0.0f;
     for (int slot = blockIdx.x * blockDim.x + threadIdx.x; slot < nslot; slot += gridDim.x * blockDim.x) {
         const int atom = p.perm[slot];
-        if (p.part != NB_PART_NONLOCAL) p.fsort[slot] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (ADJ) {
+            p.bsort[slot] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            p.gsort[slot] = atom < 0 ? make_float4(0.0f, 0.0f, 0.0f, 0.0f)
+                                     : make_float4(p.g[3 * atom], p.g[3 * atom + 1], p.g[3 * atom + 2], 0.0f);
+        } else if (p.part != NB_PART_NONLOCAL) {
+            p.fsort[slot] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
         if (atom < 0) continue;
         if (p.part == NB_PART_LOCAL ? atom >= p.n_home : (p.part == NB_PART_NONLOCAL && atom < p.n_home)) continue;
         const float4 r = p.xref[slot];
@@ -115,6 +131,8 @@ __global__ void __launch_bounds__(256) k_gather(GatherParams p) {
             for (int k = threadIdx.x; k < 2 * p.nsys; k += blockDim.x) p.energies[k] = 0.0;
         if (p.len_hist)
             for (int k = threadIdx.x; k < NB_LEN_BINS; k += blockDim.x) p.len_hist[k] = 0;
+        if (ADJ)
+            for (int k = threadIdx.x; k < p.nlj; k += blockDim.x) p.glj_acc[k] = 0.0;
     }
 }
 
@@ -384,9 +402,9 @@ int g_blocks_per_sm[3][2][2][2][2] = {};
 
 }  // namespace
 
-cudaError_t nb_launch_gather(nb_pairlist *pl, const float *coords, const float *q, const int *type,
-                             int ntype, int snapshot, double *energies, int part, cudaStream_t s) {
-    GatherParams p;
+static GatherParams gather_params(nb_pairlist *pl, const float *coords, const float *q, const int *type, int ntype,
+                                  int snapshot, double *energies, int part) {
+    GatherParams p = {};
     p.part = part;
     p.n_home = pl->n_home;
     p.ntype = ntype;
@@ -406,9 +424,28 @@ cudaError_t nb_launch_gather(nb_pairlist *pl, const float *coords, const float *
     p.len_hist = (snapshot && !(pl->flags & NB_FLAG_NO_LIST_SORT)) ? pl->len_hist : nullptr;
     p.nsys = pl->nsys;
     p.snapshot = snapshot;
-    int blocks = (pl->nc_max * NB_CLUSTER + 255) / 256;
-    blocks = max(1, min(blocks, pl->num_sms * 8));
-    return nb_launch_pdl(k_gather, blocks, 256, 0, s, p);
+    return p;
+}
+
+static int gather_blocks(const nb_pairlist *pl) {
+    return max(1, min((pl->nc_max * NB_CLUSTER + 255) / 256, pl->num_sms * 8));
+}
+
+cudaError_t nb_launch_gather(nb_pairlist *pl, const float *coords, const float *q, const int *type,
+                             int ntype, int snapshot, double *energies, int part, cudaStream_t s) {
+    const GatherParams p = gather_params(pl, coords, q, type, ntype, snapshot, energies, part);
+    return nb_launch_pdl(k_gather<false>, gather_blocks(pl), 256, 0, s, p);
+}
+
+cudaError_t nb_launch_gather_adj(nb_pairlist *pl, const float *coords, const float *q, const int *type, int ntype,
+                                 const float *g, cudaStream_t s) {
+    GatherParams p = gather_params(pl, coords, q, type, ntype, 0, nullptr, NB_PART_ALL);
+    p.g = g;
+    p.gsort = pl->gsort;
+    p.bsort = pl->bsort;
+    p.glj_acc = pl->glj_acc;
+    p.nlj = 2 * ntype * ntype;
+    return nb_launch_pdl(k_gather<true>, gather_blocks(pl), 256, 0, s, p);
 }
 
 cudaError_t nb_launch_force(nb_pairlist *pl, int ntype, const float *ljparams, float rc, float beta,

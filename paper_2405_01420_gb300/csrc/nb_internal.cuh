@@ -251,6 +251,9 @@ cudaError_t nb_launch_search(nb_pairlist *pl, const int *excl_off, const int *ex
 // lists are sorted, clears the list-length histogram).
 cudaError_t nb_launch_gather(nb_pairlist *pl, const float *coords, const float *q, const int *type,
                              int ntype, int snapshot, double *energies, int part, cudaStream_t s);
+// The gather of an adjoint call: also g = dL/dF to cluster order, and zeroed adjoint accumulators.
+cudaError_t nb_launch_gather_adj(nb_pairlist *pl, const float *coords, const float *q, const int *type, int ntype,
+                                 const float *g, cudaStream_t s);
 // clus_home[c] bit b = slot b of cluster c holds a home atom (after the grid sort of a search).
 cudaError_t nb_launch_clus_home(nb_pairlist *pl, cudaStream_t s);
 cudaError_t nb_launch_prune(nb_pairlist *pl, float r_inner2, float stale_search2, cudaStream_t s);
@@ -277,5 +280,4 @@ cudaError_t nb_launch_force(nb_pairlist *pl, int ntype, const float *ljparams, f
                             cudaStream_t s);
 cudaError_t nb_launch_scatter(nb_pairlist *pl, float *forces, cudaStream_t s);
 cudaError_t nb_launch_backward(nb_pairlist *pl, int ntype, const float *ljparams, float rc, float beta,
-                               const float *g, float *grad_x, float *grad_q, double *grad_lj,
-                               float stale_search2, float stale_prune2, cudaStream_t s);
+                               float *grad_x, float *grad_q, double *grad_lj, float stale_search2, float stale_prune2, cudaStream_t s);
