@@ -101,63 +101,95 @@ __device__ __forceinline__ void pme_offsets(const pme_axes &ax, const int base[3
     if (zc < 0) zc += ax.K[2];
 }
 
+// Clears the mesh ahead of the spread, which starts (with programmatic
+// dependent launch) while this runs. Launched the usual way, so everything
+// before it in the stream has completed by then.
+__global__ void __launch_bounds__(kThreads) k_pme_clear(float *__restrict__ grid, unsigned cells) {
+    nb_pdl_release();
+    const unsigned t = blockIdx.x * kThreads + threadIdx.x, stride = gridDim.x * kThreads;
+    if (((size_t)grid & 15u) == 0) {
+        for (unsigned k = t; k < cells / 4; k += stride) reinterpret_cast<float4 *>(grid)[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (t < (cells & 3u)) grid[(cells & ~3u) + t] = 0.0f;
+    } else {
+        for (unsigned k = t; k < cells; k += stride) grid[k] = 0.0f;
+    }
+}
+
+// A lane's part of one atom's support: x and y weights with the mesh offsets
+// of their planes and rows, and the charge times the weight of its z point.
+struct pme_part {
+    float mx[4], my[4], v;
+    int xo[4], yo[4], zc;
+};
+
+__device__ __forceinline__ pme_part pme_load(unsigned i, int c, const float *__restrict__ coords,
+                                             const float *__restrict__ q, const pme_axes &ax) {
+    const float *xi = coords + 3 * (size_t)i;
+    pme_part r;
+    float w[3], mz[4];
+    int base[3];
+    const float qi = __ldg(q + i);
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+        pme_scaled(__ldg(xi + a), ax.s_hi[a], ax.s_lo[a], ax.Kf[a], ax.invK[a], ax.K[a], w[a], base[a]);
+    pme_w4(w[0], r.mx);
+    pme_w4(w[1], r.my);
+    pme_w4(w[2], mz);
+    r.v = qi * pme_pick(mz, c);
+    pme_offsets(ax, base, c, r.xo, r.yo, r.zc);
+    return r;
+}
+
+// Each thread's first atom is read and its weights are formed before the wait
+// for the cleared mesh.
 __global__ void __launch_bounds__(kThreads) k_pme_spread(int n, const float *__restrict__ coords,
                                                          const float *__restrict__ q, pme_axes ax,
                                                          float *__restrict__ grid) {
     const int c = threadIdx.x & (kLanesPerAtom - 1);
     // unsigned: n < 2^31 and the stride is below 2^17, so i + stride never wraps
     const unsigned stride = gridDim.x * (kThreads / kLanesPerAtom);
-    for (unsigned i = blockIdx.x * (kThreads / kLanesPerAtom) + (threadIdx.x >> 2); i < (unsigned)n; i += stride) {
-        const float qi = __ldg(q + i);
-        const float *xi = coords + 3 * (size_t)i;
-        float w[3];
-        int base[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-            pme_scaled(__ldg(xi + a), ax.s_hi[a], ax.s_lo[a], ax.Kf[a], ax.invK[a], ax.K[a], w[a],
-                       base[a]);
-        float mx[4], my[4], mz[4];
-        pme_w4(w[0], mx);
-        pme_w4(w[1], my);
-        pme_w4(w[2], mz);
-        const float v = qi * pme_pick(mz, c);
-        int xo[4], yo[4], zc;
-        pme_offsets(ax, base, c, xo, yo, zc);
+    unsigned i = blockIdx.x * (kThreads / kLanesPerAtom) + (threadIdx.x >> 2);
+    pme_part r;
+    if (i < (unsigned)n) r = pme_load(i, c, coords, q, ax);
+    nb_pdl_wait();
+    while (i < (unsigned)n) {
 #pragma unroll
         for (int a = 0; a < kOrder; ++a) {
-            const float va = v * mx[a];
+            const float va = r.v * r.mx[a];
 #pragma unroll
-            for (int b = 0; b < kOrder; ++b) atomicAdd(grid + (xo[a] + yo[b] + zc), va * my[b]);
+            for (int b = 0; b < kOrder; ++b) atomicAdd(grid + (r.xo[a] + r.yo[b] + r.zc), va * r.my[b]);
         }
+        i += stride;
+        if (i < (unsigned)n) r = pme_load(i, c, coords, q, ax);
     }
 }
 
+// After the four sums over an atom's 4 lanes, one component per lane: lane 0
+// x, 1 y, 2 z of the force, 3 the potential. Without the energy there is no
+// FP64 operation (the FP64 pipe takes 16 cycles per warp instruction and SM).
+template <bool ENERGY>
 __global__ void __launch_bounds__(kThreads) k_pme_gather(int n, const float *__restrict__ coords,
                                                          const float *__restrict__ q, pme_axes ax,
                                                          const float *__restrict__ phi, float *__restrict__ forces,
                                                          int accumulate, double *__restrict__ energy) {
     const int c = threadIdx.x & (kLanesPerAtom - 1);
-    const long long stride = (long long)gridDim.x * (kThreads / kLanesPerAtom);
+    const int first = (threadIdx.x & 31) >> 2;  // the lane's atom among the warp's 8
+    // unsigned: n < 2^31 and the stride is below 2^17, so i0 + stride never wraps
+    const unsigned stride = gridDim.x * (kThreads / kLanesPerAtom);
     double e_acc = 0.0;
-    // every lane group runs the same number of iterations, so the shuffles below see all 32 lanes
-    const long long n_round = ((long long)n + stride - 1) / stride * stride;
-    for (long long i = (long long)blockIdx.x * (kThreads / kLanesPerAtom) + (threadIdx.x >> 2); i < n_round;
-         i += stride) {
-        const bool live = i < n;
+    // i0, the warp's first atom, is the same in all lanes, so the shuffles below see all 32
+    for (unsigned i0 = (blockIdx.x * kThreads + (threadIdx.x & ~31u)) / kLanesPerAtom; i0 < (unsigned)n; i0 += stride) {
+        const unsigned i = i0 + first;
+        const bool live = i < (unsigned)n;
         float psi = 0.0f, gx = 0.0f, gy = 0.0f, gz = 0.0f, qi = 0.0f;
         if (live) {
             qi = __ldg(q + i);
+            const float *xi = coords + 3 * (size_t)i;
             float w[3];
             int base[3];
 #pragma unroll
             for (int a = 0; a < 3; ++a)
-                pme_scaled(__ldg(coords + 3 * i + a), ax.s_hi[a], ax.s_lo[a], ax.Kf[a], ax.invK[a], ax.K[a], w[a],
-                           base[a]);
-            float mx[4], dx[4], my[4], dy[4];
-            pme_w4(w[0], mx);
-            pme_d4(w[0], dx);
-            pme_w4(w[1], my);
-            pme_d4(w[1], dy);
+                pme_scaled(__ldg(xi + a), ax.s_hi[a], ax.s_lo[a], ax.Kf[a], ax.invK[a], ax.K[a], w[a], base[a]);
             int xo[4], yo[4], zc;
             pme_offsets(ax, base, c, xo, yo, zc);
             float p[kOrder][kOrder];
@@ -165,6 +197,11 @@ __global__ void __launch_bounds__(kThreads) k_pme_gather(int n, const float *__r
             for (int a = 0; a < kOrder; ++a)
 #pragma unroll
                 for (int b = 0; b < kOrder; ++b) p[a][b] = __ldg(phi + (xo[a] + yo[b] + zc));
+            float mx[4], dx[4], my[4], dy[4];
+            pme_w4(w[0], mx);
+            pme_d4(w[0], dx);
+            pme_w4(w[1], my);
+            pme_d4(w[1], dy);
             float s_m = 0.0f, s_dx = 0.0f, s_dy = 0.0f;  // sums over the lane's 16 (x, y) points
 #pragma unroll
             for (int a = 0; a < kOrder; ++a) {
@@ -187,21 +224,25 @@ __global__ void __launch_bounds__(kThreads) k_pme_gather(int n, const float *__r
             gy = mz * s_dy;
             gz = dz * s_m;
         }
-#pragma unroll
-        for (int o = 1; o < kLanesPerAtom; o <<= 1) {
-            psi += __shfl_xor_sync(0xffffffffu, psi, o);
-            gx += __shfl_xor_sync(0xffffffffu, gx, o);
-            gy += __shfl_xor_sync(0xffffffffu, gy, o);
-            gz += __shfl_xor_sync(0xffffffffu, gz, o);
-        }
-        if (live && c == 0) {
-            const float f[3] = {-qi * ax.s[0] * gx, -qi * ax.s[1] * gy, -qi * ax.s[2] * gz};
-#pragma unroll
-            for (int a = 0; a < 3; ++a) forces[3 * i + a] = accumulate ? forces[3 * i + a] + f[a] : f[a];
-            e_acc += 0.5 * (double)qi * (double)psi;
+        // sum over the atom's 4 lanes: first over lane ^ 1 (even lanes go on with gx and gz, odd ones
+        // with gy and psi), then over lane ^ 2
+        const bool odd = c & 1, high = c & 2;
+        float u = odd ? gy : gx, v = odd ? psi : gz;
+        u += __shfl_xor_sync(0xffffffffu, odd ? gx : gy, 1);
+        v += __shfl_xor_sync(0xffffffffu, odd ? gz : psi, 1);
+        float r = high ? v : u;
+        r += __shfl_xor_sync(0xffffffffu, high ? u : v, 2);
+        if (live) {
+            if (c < 3) {
+                const float f = -qi * (c == 0 ? ax.s[0] : c == 1 ? ax.s[1] : ax.s[2]) * r;
+                float *out = forces + 3 * (size_t)i + c;
+                *out = accumulate ? *out + f : f;
+            } else if (ENERGY) {
+                e_acc += 0.5 * (double)qi * (double)r;
+            }
         }
     }
-    if (energy) {
+    if (ENERGY) {
 #pragma unroll
         for (int o = 16; o >= 1; o >>= 1) e_acc += __shfl_xor_sync(0xffffffffu, e_acc, o);
         if ((threadIdx.x & 31) == 0 && e_acc != 0.0) atomicAdd(energy, e_acc);
@@ -250,10 +291,11 @@ int pme_check(const char *who, int n, const float *coords, const float *q, const
 
 // One wave of resident blocks (the kernels stride over the atoms), or fewer
 // for a small system. The SM count and the kernel's occupancy are looked up
-// once per device and kernel (kind 0 spread, 1 gather).
+// once per device and kernel (kind 0 spread, 1 gather, 2 gather with
+// energy).
 constexpr int kMaxDevices = 64;
 int g_pme_sms[kMaxDevices] = {};
-int g_pme_per_sm[kMaxDevices][2] = {};
+int g_pme_per_sm[kMaxDevices][3] = {};
 
 int pme_blocks(int n, const void *kernel, int kind) {
     int dev = 0;
@@ -282,12 +324,13 @@ extern "C" int nb_pme_spread(int n_atoms, const float *coords, const float *q, c
     if (rc != NB_OK) return rc;
     if (!grid) return nb_record_error(NB_ERR_ARG, "nb_pme_spread: NULL grid");
     cudaStream_t s = (cudaStream_t)stream;
-    const size_t cells = (size_t)K0 * K1 * K2;
-    cudaError_t e = cudaMemsetAsync(grid, 0, sizeof(float) * cells, s);
-    if (e == cudaSuccess && n_atoms > 0) {
-        k_pme_spread<<<pme_blocks(n_atoms, (const void *)k_pme_spread, 0), kThreads, 0, s>>>(n_atoms, coords, q, ax, grid);
-        e = cudaGetLastError();
-    }
+    const unsigned cells = (unsigned)((size_t)K0 * K1 * K2);
+    constexpr unsigned per_block = 16 * kThreads;
+    k_pme_clear<<<(cells + per_block - 1) / per_block, kThreads, 0, s>>>(grid, cells);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess && n_atoms > 0)
+        e = nb_launch_pdl(k_pme_spread, pme_blocks(n_atoms, (const void *)k_pme_spread, 0), kThreads, 0, s, n_atoms,
+                          coords, q, ax, grid);
     if (e != cudaSuccess) return nb_record_error(NB_ERR_CUDA, cudaGetErrorString(e));
     return NB_OK;
 }
@@ -303,7 +346,8 @@ extern "C" int nb_pme_gather(int n_atoms, const float *coords, const float *q, c
     cudaError_t e = cudaSuccess;
     if (energy) e = cudaMemsetAsync(energy, 0, sizeof(double), s);
     if (e == cudaSuccess && n_atoms > 0) {
-        k_pme_gather<<<pme_blocks(n_atoms, (const void *)k_pme_gather, 1), kThreads, 0, s>>>(
+        const auto kernel = energy ? k_pme_gather<true> : k_pme_gather<false>;
+        kernel<<<pme_blocks(n_atoms, (const void *)kernel, energy ? 2 : 1), kThreads, 0, s>>>(
             n_atoms, coords, q, ax, phi, forces, accumulate ? 1 : 0, energy);
         e = cudaGetLastError();
     }
