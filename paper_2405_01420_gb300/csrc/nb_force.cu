@@ -109,12 +109,22 @@ __global__ void __launch_bounds__(256) k_gather(GatherParams p) {
             d2p_max = fmaxf(d2p_max, ex * ex + ey * ey + ez * ez);
         }
     }
+    // One atomic per block and maximum: atomics on one address are served one per 1.3 ns, and one per
+    // warp held the kernel at 8.8 us for 96,000 atoms
+    __shared__ float s_max[2][256 / 32];
     d2s_max = warp_max(d2s_max);
     d2p_max = warp_max(d2p_max);
     if ((threadIdx.x & 31) == 0) {
+        s_max[0][threadIdx.x >> 5] = d2s_max;
+        s_max[1][threadIdx.x >> 5] = d2p_max;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        float m = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 256 / 32; ++k) m = fmaxf(m, s_max[threadIdx.x][k]);
         // non-negative floats order like their bit patterns
-        if (d2s_max > 0.0f) atomicMax(&p.st->cur_d2_search, __float_as_uint(d2s_max));
-        if (d2p_max > 0.0f) atomicMax(&p.st->cur_d2_prune, __float_as_uint(d2p_max));
+        if (m > 0.0f) atomicMax(threadIdx.x == 0 ? &p.st->cur_d2_search : &p.st->cur_d2_prune, __float_as_uint(m));
     }
     if (blockIdx.x == 0) {
         if (threadIdx.x == 0) {
