@@ -130,6 +130,9 @@ __global__ void __launch_bounds__(kPruneThreads, kPruneCtasPerSm) k_prune(PruneP
     // 16-byte reads of one atom index free of bank conflicts
     __shared__ float4 s_xj[kPruneWarps][32][NB_CLUSTER + 1];
     __shared__ uint2 s_ring[kPruneWarps][kSets][kStage];  // staged atoms: (slot word, entry's mask word)
+    __shared__ unsigned s_total[2], s_done;  // the CTA's kept entries and gathered tiles; its finished warps
+    if (threadIdx.x == 0) s_total[0] = s_total[1] = s_done = 0u;
+    __syncthreads();
     nb_pdl_wait();  // launched with nb_launch_pdl: the prune's gather has completed from here on
     nb_pdl_release();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -144,14 +147,17 @@ __global__ void __launch_bounds__(kPruneThreads, kPruneCtasPerSm) k_prune(PruneP
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lanebit = 1u << lane;
     const int nc = p.st->nc;
-    const unsigned nwarps = gridDim.x * kPruneWarps;
-    for (unsigned it = 0;; ++it) {
-        // a warp's first i-cluster is its own index in the grid, later ones come from the counter
-        unsigned w = blockIdx.x * kPruneWarps + warp;
-        if (it > 0) {
-            unsigned a = 0;
-            if (lane == 0) a = atomicAdd(&p.st->work_prune, 1u);
-            w = __shfl_sync(0xffffffffu, a, 0) + nwarps;
+    const unsigned nwarps = gridDim.x * kPruneWarps, run = ticket_run((unsigned)nc, nwarps);
+    unsigned w = 0u, end = 0u;
+    for (bool first = true;; first = false) {
+        if (++w >= end) {
+            // a warp's first ticket is its own index in the grid, later ones come from the counter
+            unsigned k = blockIdx.x * kPruneWarps + warp;
+            if (!first) {
+                if (lane == 0) k = atomicAdd(&p.st->work_prune, 1u);
+                k = __shfl_sync(0xffffffffu, k, 0) + nwarps;
+            }
+            ticket_items(k, (unsigned)nc, run, w, end);
         }
         if (w >= (unsigned)nc) break;
         const int ci = (int)w;
@@ -305,17 +311,27 @@ __global__ void __launch_bounds__(kPruneThreads, kPruneCtasPerSm) k_prune(PruneP
         __syncwarp();
         if (lane == 0) {
             p.ci_len_inner[ci] = out;
-            atomicAdd(&p.st->inner_count, (unsigned long long)out);
+            atomicAdd(&s_total[0], (unsigned)out);
             // post-prune sorting: the force kernel's work for ci and its histogram
             int key = out;
             if (TILES) {
                 key = 0;
 #pragma unroll
                 for (int r = 0; r < kSets; ++r) key += ntile[r];
-                atomicAdd(&p.st->tile_count, (unsigned long long)key);
+                atomicAdd(&s_total[1], (unsigned)key);
             }
             p.len_key[ci] = key;
             if (p.len_hist) atomicAdd(&p.len_hist[min(key, NB_LEN_BINS - 1)], 1);
+        }
+    }
+    // the CTA's totals, from its last warp: two atomics per i-cluster on these addresses (with the
+    // counter and the histogram 4, one per 1.3 ns) were what bounded the kernel
+    if (lane == 0) {
+        __threadfence_block();
+        if (atomicAdd(&s_done, 1u) == kPruneWarps - 1) {
+            __threadfence_block();
+            atomicAdd(&p.st->inner_count, (unsigned long long)atomicAdd(&s_total[0], 0u));
+            if (TILES) atomicAdd(&p.st->tile_count, (unsigned long long)atomicAdd(&s_total[1], 0u));
         }
     }
 }

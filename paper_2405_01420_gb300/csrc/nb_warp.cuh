@@ -1,5 +1,6 @@
 // Warp-level helpers of the gathered-tile kernels: asynchronous copies into
-// shared memory and a reduce-scatter of per-lane partial sums.
+// shared memory, a reduce-scatter of per-lane partial sums, the order in
+// which persistent warps take their work.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -46,3 +47,17 @@ __device__ __forceinline__ void reduce_scatter(float (&v)[N], int lane) {
 #pragma unroll
     for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
 }
+
+// Work items handed out by a counter. Ticket k stands for the items [a, b):
+// the first three quarters of the n items go in runs of `run`, the rest one
+// by one, so that the launch still ends with single items. Atomics on one
+// address are served one per 1.3 ns, too slowly for a ticket per short item.
+__device__ __forceinline__ void ticket_items(unsigned k, unsigned n, unsigned run, unsigned &a, unsigned &b) {
+    const unsigned runs = run > 1u ? (n - n / 4u) / run : 0u;
+    const bool in_run = k < runs;
+    a = in_run ? k * run : runs * run + (k - runs);
+    b = a + (in_run ? run : 1u);
+}
+
+// Items per run for nwarps warps: at least 6 runs for each warp.
+__device__ __forceinline__ unsigned ticket_run(unsigned n, unsigned nwarps) { return min(max(n / (8u * nwarps), 1u), 8u); }
