@@ -12,9 +12,12 @@
 //    kept in shared memory, a row pair's four in one float4 of the lane's
 //    own column (any 8 lanes cover the 32 banks whatever their types),
 //    reduced across the warp once per half by a skewed read (lane k sums
-//    value k, starting at column k) and added in FP64 to the unsymmetrised
-//    [ntype][ntype][2] accumulator. In registers they took 32 of them and
-//    held the kernel at 4 warps per scheduler.
+//    value k, starting at column k) and added in FP64 to the warp's
+//    [ntype][ntype][2] sums, which each CTA adds to the unsymmetrised
+//    accumulator at its end (from every half, these atomics on a few sectors
+//    were served too slowly: they, not the pairs, set the kernel's time). In
+//    registers the FP32 accumulators took 32 of them and held the kernel at 4
+//    warps per scheduler.
 // Group g + 1's j data (coordinates and charge, g, type, mask word) are
 // loaded into registers while group g is computed, their slot words one
 // group earlier still; groups at the center image skip S = 0; halves are
@@ -94,6 +97,8 @@ __global__ void __launch_bounds__(kBvtThreads, kBvtCtasPerSm) k_backward_vt(BvtP
     extern __shared__ float4 s_lj[];
     // per warp, row pair k, j type and lane: (C6 of row 2k, C12 of row 2k, C6 of row 2k + 1, C12 of row 2k + 1)
     __shared__ float4 s_acc[kBvtWarps][2 * NT][32];
+    __shared__ double s_glj[kBvtWarps][2 * NT * NT];  // the warp's LJ gradients, [type][type][C6 / C12]
+    __shared__ unsigned s_done;  // finished warps
     __shared__ float4 s_shift[kBvtWarps][27];
     __shared__ float4 s_xi[kBvtWarps][4];  // (x, y, z, f q)
     __shared__ float4 s_gi[kBvtWarps][4];
@@ -105,6 +110,7 @@ __global__ void __launch_bounds__(kBvtThreads, kBvtCtasPerSm) k_backward_vt(BvtP
     const int nt2 = p.ntype * p.ntype;
     for (int k = threadIdx.x; k < nt2; k += blockDim.x)
         s_lj[k] = make_float4(p.ljparams[2 * k], p.ljparams[2 * k + 1], 0.0f, 0.0f);
+    if (threadIdx.x == 0) s_done = 0u;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const unsigned ds = p.st->cur_d2_search, dp = p.st->cur_d2_prune;
         p.st->last_d2_search = ds;
@@ -122,6 +128,8 @@ __global__ void __launch_bounds__(kBvtThreads, kBvtCtasPerSm) k_backward_vt(BvtP
     float4(*acc)[32] = s_acc[warp];
 #pragma unroll
     for (int k = 0; k < 2 * NT; ++k) acc[k][lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (lane < 2 * NT * NT) s_glj[warp][lane] = 0.0;
+    __syncwarp();
 
     const unsigned nwarps = gridDim.x * kBvtWarps;
     for (unsigned it = 0;; ++it) {
@@ -256,18 +264,35 @@ __global__ void __launch_bounds__(kBvtThreads, kBvtCtasPerSm) k_backward_vt(BvtP
         // LJ gradients: value k = (a NT + t) 2 + c, summed over the 32 columns by lane k, which starts
         // at column k (4 lanes meet in the banks of a column, two of them in the same word)
         __syncwarp();
+        const int a = lane / (2 * NT), t = (lane >> 1) % NT, c = lane & 1;
+        float sum = 0.0f;
         if (lane < kAcc) {
-            const int a = lane / (2 * NT), t = (lane >> 1) % NT, c = lane & 1;
             const float *val = reinterpret_cast<const float *>(acc[(a >> 1) * NT + t]) + 2 * (a & 1) + c;
-            float sum = 0.0f;
 #pragma unroll 8
             for (int i = 0; i < 32; ++i) sum += val[4 * ((i + lane) & 31)];
-            if (t < p.ntype && sum != 0.0f) atomicAdd(&p.glj_acc[2 * (s_tr[warp][a] + t) + c], (double)sum);
+        }
+#pragma unroll
+        for (int row = 0; row < 4; ++row) {  // one row at a time: rows of one type share their sums
+            if (a == row && t < p.ntype) s_glj[warp][2 * (s_tr[warp][row] + t) + c] += (double)sum;
+            __syncwarp();
         }
         __syncwarp();
 #pragma unroll
         for (int k = 0; k < 2 * NT; ++k) acc[k][lane] = make_float4(0.f, 0.f, 0.f, 0.f);
         __syncwarp();
+    }
+    // the CTA's LJ gradients, from its last warp
+    unsigned done = 0u;
+    if (lane == 0) {
+        __threadfence_block();
+        done = atomicAdd(&s_done, 1u);
+        __threadfence_block();
+    }
+    if (__shfl_sync(0xffffffffu, done, 0) == kBvtWarps - 1 && lane < 2 * nt2) {
+        double sum = 0.0;
+#pragma unroll
+        for (int k = 0; k < kBvtWarps; ++k) sum += *(volatile double *)&s_glj[k][lane];
+        if (sum != 0.0) atomicAdd(&p.glj_acc[lane], sum);
     }
 }
 
