@@ -162,6 +162,7 @@ int alloc_pairlist(nb_pairlist *pl, long long n, const nb_config *cfg, const cha
     if (!pl->sys_host) return fail(NB_ERR_NOMEM, "%s: host allocation failed", who);
     // Defined contents for everything a kernel may read before the first search writes it.
     NB_CUDA(cudaMemset(pl->st, 0, sizeof(nb_dev_state)));
+    NB_CUDA(cudaMemset(pl->col_count, 0, sizeof(int) * (size_t)pl->ncol_max));
     NB_CUDA(cudaMemset(pl->pos, 0, sizeof(int) * (size_t)n));
     NB_CUDA(cudaMemset(pl->perm, 0xff, sizeof(int) * nslot));
     NB_CUDA(cudaMemset(pl->ci_start, 0, sizeof(int) * (size_t)pl->nc_max));
@@ -315,7 +316,7 @@ extern "C" int nb_search(nb_pairlist *pl, const float *coords, const float *box,
         pl->ncol = ncx * ncy;
         pl->sys_host[0] = make_sys(box, ncx, ncy, 0, 0, pl->n_atoms);
     }
-    // the grid sort's first kernel clears the list counter (and writes a single system's table)
+    // the grid sort's first kernel clears the list counter and writes a single system's table
     NB_CUDA(nb_launch_grid_sort(pl, coords, pl->batch ? nullptr : &pl->sys_host[0], s));
 
     // The bounding-box test uses a radius inflated by a few ulps of the box

@@ -1,15 +1,16 @@
 // Grid sort into 8-atom clusters (first stage of the pair search, §III-A).
 //
-// 0. k_search_begin: clear the column counts and the list counter; write a
-//    single system's table.
 // 1. k_bin: wrap each atom into the box and bin it into an xy column;
-//    count atoms per column.
+//    count atoms per column. Also writes a single system's table.
 // 2. k_col_scan: exclusive scans of atoms and of 8-atom clusters per column.
-// 3. k_col_scatter: bucket (z, atom) keys by column.
+// 3. k_col_scatter: bucket (z, atom) keys by column. With few columns each of
+//    its blocks makes the scan for itself, and 2 is left out.
 // 4. k_col_sort: sorts each column's keys by z (bitonic: in one warp's
 //    registers up to 256 atoms, else by a CTA in shared memory), packs runs
 //    of 8 into clusters, pads the last one, and writes the slot <-> atom
-//    maps, the search-frame positions and per-cluster bounding boxes.
+//    maps, the search-frame positions and per-cluster bounding boxes. Clears
+//    the column counts, which are 0 between searches: a kernel of its own for
+//    that, at the start, cost a search of a small box 2 us.
 //
 // Layout in HBM after the sort (slot = 8 * cluster + lane):
 //   perm[slot] (int), xref[slot] (float4), bbox[2c], bbox[2c+1] (float4).
@@ -20,37 +21,31 @@
 
 namespace {
 
-// The start of a search: clears the column counts and the list counter and,
-// for a single-system pair list, writes its system table (one entry and its
-// 27 shift vectors) from kernel arguments, so that a search can be captured
-// in a CUDA graph without a host-to-device copy. Like every kernel of the
-// grid sort and the search it may be launched with programmatic dependent
-// launch (nb_launch_if, for lists up to NB_SEARCH_PDL_MAX_CLUSTERS).
-__global__ void k_search_begin(nb_sys *sys, float4 *sys_shift, nb_sys one, int write_sys, int *col_count, int ncol,
-                               nb_dev_state *st) {
-    nb_pdl_wait();
-    nb_pdl_release();
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < ncol; k += gridDim.x * blockDim.x) col_count[k] = 0;
-    if (blockIdx.x != 0) return;
-    const int k = threadIdx.x;
-    if (k == 0) st->list_count = 0ull;
-    if (!write_sys) return;
-    if (k == 0) sys[0] = one;
-    if (k < 27)
-        sys_shift[k] = make_float4((float)nb_shift_x(k) * one.box.x, (float)nb_shift_y(k) * one.box.y,
-                                   (float)nb_shift_z(k) * one.box.z, 0.0f);
-}
-
+// one: a single-system list's table (one entry and its 27 shift vectors),
+// which comes in the kernel arguments, so that a search can be captured in a
+// CUDA graph without a host-to-device copy; a batch's is uploaded when it is
+// created. Like every kernel of the grid sort and the search this one may be
+// launched with programmatic dependent launch (nb_launch_if, for lists up to
+// NB_SEARCH_PDL_MAX_CLUSTERS).
 __global__ void k_bin(int n, const float *__restrict__ coords, const int *__restrict__ atom_sys,
-                      const nb_sys *__restrict__ sys, int *__restrict__ col_count, int *__restrict__ atom_col,
-                      int *__restrict__ atom_slot, float4 *__restrict__ xw, nb_dev_state *st) {
+                      nb_sys *sys, float4 *sys_shift, nb_sys one, int single, int *__restrict__ col_count,
+                      int *__restrict__ atom_col, int *__restrict__ atom_slot, float4 *__restrict__ xw,
+                      nb_dev_state *st) {
     nb_pdl_wait();
     nb_pdl_release();
+    if (blockIdx.x == 0) {
+        const int k = threadIdx.x;
+        if (k == 0) st->list_count = 0ull;
+        if (single && k == 0) sys[0] = one;
+        if (single && k < 27)
+            sys_shift[k] = make_float4((float)nb_shift_x(k) * one.box.x, (float)nb_shift_y(k) * one.box.y,
+                                       (float)nb_shift_z(k) * one.box.z, 0.0f);
+    }
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
     int col = -1 - lane;  // lanes past the end match nobody below
     if (i < n) {
-        const nb_sys S = sys[atom_sys[i]];
+        const nb_sys S = single ? one : sys[atom_sys[i]];
         float x = coords[3 * i + 0], y = coords[3 * i + 1], z = coords[3 * i + 2];
         if (!(isfinite(x) && isfinite(y) && isfinite(z))) {
             atomicOr(&st->err, NB_DEV_NONFINITE);
@@ -76,8 +71,77 @@ __global__ void k_bin(int n, const float *__restrict__ coords, const int *__rest
     if (i < n) atom_slot[i] = base + __popc(peers & ((1u << lane) - 1u));
 }
 
-// Single CTA: exclusive scans of col_count (atoms) and ceil(count/8)
-// (clusters) over ncol columns; total clusters -> st->nc.
+constexpr int kScanPerThread = 4;  // consecutive columns per thread and pass of a scan
+constexpr int kScatterThreads = 256;
+constexpr int kScanInScatter = kScanPerThread * kScatterThreads;  // columns a block of the scatter scans itself
+
+// Exclusive scans of col_count (atoms) and ceil(count/8) (clusters) over ncol
+// columns by one CTA; out(c, atoms before, clusters before) for each column
+// and, from thread 0, for c = ncol. Returns whether a column of this thread
+// holds too many atoms.
+template <typename Out>
+__device__ __forceinline__ bool scan_columns(int ncol, const int *__restrict__ col_count, int *warp_a, int *warp_c,
+                                             Out out) {
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5, nw = blockDim.x >> 5;
+    int carry_a = 0, carry_c = 0;
+    bool over = false;
+    for (int c0 = 0; c0 < ncol; c0 += kScanPerThread * blockDim.x) {
+        const int c = c0 + kScanPerThread * t;
+        // Atom offsets use the full counts (every atom gets a key slot); cluster
+        // offsets use the counts the per-column sort can hold, so that every
+        // allocated cluster slot is written even after a column overflow.
+        int ka[kScanPerThread], kc[kScanPerThread], sa = 0, sc = 0;
+#pragma unroll
+        for (int j = 0; j < kScanPerThread; ++j) {
+            ka[j] = c + j < ncol ? col_count[c + j] : 0;
+            kc[j] = (min(ka[j], NB_MAX_COL_ATOMS) + NB_CLUSTER - 1) / NB_CLUSTER;
+            over |= ka[j] > NB_MAX_COL_ATOMS;
+            sa += ka[j];
+            sc += kc[j];
+        }
+        // inclusive scan of (sa, sc) across the CTA
+        int ia = sa, ic = sc;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int va = __shfl_up_sync(0xffffffffu, ia, o), vc = __shfl_up_sync(0xffffffffu, ic, o);
+            if (lane >= o) {
+                ia += va;
+                ic += vc;
+            }
+        }
+        __syncthreads();  // the previous pass's reads of warp_a, warp_c are over
+        if (lane == 31) {
+            warp_a[wid] = ia;
+            warp_c[wid] = ic;
+        }
+        __syncthreads();
+        // every warp scans the warps' totals itself
+        int wa = lane < nw ? warp_a[lane] : 0, wc = lane < nw ? warp_c[lane] : 0;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int va = __shfl_up_sync(0xffffffffu, wa, o), vc = __shfl_up_sync(0xffffffffu, wc, o);
+            if (lane >= o) {
+                wa += va;
+                wc += vc;
+            }
+        }
+        const int ba = __shfl_sync(0xffffffffu, wa, max(wid - 1, 0)), bc = __shfl_sync(0xffffffffu, wc, max(wid - 1, 0));
+        int pa = carry_a + (wid > 0 ? ba : 0) + ia - sa;  // exclusive prefix of this thread
+        int pc = carry_c + (wid > 0 ? bc : 0) + ic - sc;
+        carry_a += __shfl_sync(0xffffffffu, wa, 31);
+        carry_c += __shfl_sync(0xffffffffu, wc, 31);
+#pragma unroll
+        for (int j = 0; j < kScanPerThread; ++j) {
+            if (c + j < ncol) out(c + j, pa, pc);
+            pa += ka[j];
+            pc += kc[j];
+        }
+    }
+    if (t == 0) out(ncol, carry_a, carry_c);
+    return over;
+}
+
+// Single CTA: the scans; total clusters -> st->nc. (With one chunk of
+// columns per thread its reads were not coalesced: 43 us for the 35,000
+// columns of a 256-box batch.)
 __global__ void __launch_bounds__(1024) k_col_scan(int ncol, const int *__restrict__ col_count,
                                                    int *__restrict__ col_atom_start,
                                                    int *__restrict__ col_clus_start,
@@ -85,80 +149,50 @@ __global__ void __launch_bounds__(1024) k_col_scan(int ncol, const int *__restri
     nb_pdl_wait();
     nb_pdl_release();
     __shared__ int warp_a[32], warp_c[32];
-    int t = threadIdx.x, nt = blockDim.x;
-    int chunk = (ncol + nt - 1) / nt;
-    int b = t * chunk, e = min(ncol, b + chunk);
-    int sa = 0, sc = 0, over = 0;
-    // Atom offsets use the full counts (every atom gets a key slot); cluster
-    // offsets use the counts the per-column sort can hold, so that every
-    // allocated cluster slot is written even after a column overflow.
-    for (int c = b; c < e; ++c) {
-        int k = col_count[c];
-        sa += k;
-        sc += (min(k, NB_MAX_COL_ATOMS) + NB_CLUSTER - 1) / NB_CLUSTER;
-        over |= (k > NB_MAX_COL_ATOMS);
-    }
+    const bool over = scan_columns(ncol, col_count, warp_a, warp_c, [&](int c, int a, int k) {
+        col_atom_start[c] = a;
+        col_clus_start[c] = k;
+        if (c == ncol) st->nc = k;
+    });
     if (over) atomicOr(&st->err, NB_DEV_COLUMN_OVERFLOW);
-    // inclusive scan of (sa, sc) across the CTA
-    int lane = t & 31, wid = t >> 5;
-    int ia = sa, ic = sc;
-    for (int o = 1; o < 32; o <<= 1) {
-        int va = __shfl_up_sync(0xffffffffu, ia, o), vc = __shfl_up_sync(0xffffffffu, ic, o);
-        if (lane >= o) {
-            ia += va;
-            ic += vc;
-        }
-    }
-    if (lane == 31) {
-        warp_a[wid] = ia;
-        warp_c[wid] = ic;
-    }
-    __syncthreads();
-    if (wid == 0) {
-        int nw = nt >> 5;
-        int va = lane < nw ? warp_a[lane] : 0, vc = lane < nw ? warp_c[lane] : 0;
-        for (int o = 1; o < 32; o <<= 1) {
-            int ua = __shfl_up_sync(0xffffffffu, va, o), uc = __shfl_up_sync(0xffffffffu, vc, o);
-            if (lane >= o) {
-                va += ua;
-                vc += uc;
-            }
-        }
-        warp_a[lane] = va;
-        warp_c[lane] = vc;
-    }
-    __syncthreads();
-    int pa = (wid > 0 ? warp_a[wid - 1] : 0) + ia - sa;  // exclusive prefix of this thread
-    int pc = (wid > 0 ? warp_c[wid - 1] : 0) + ic - sc;
-    for (int c = b; c < e; ++c) {
-        col_atom_start[c] = pa;
-        col_clus_start[c] = pc;
-        int k = col_count[c];
-        pa += k;
-        pc += (min(k, NB_MAX_COL_ATOMS) + NB_CLUSTER - 1) / NB_CLUSTER;
-    }
-    if (t == nt - 1) {
-        col_atom_start[ncol] = pa;
-        col_clus_start[ncol] = pc;
-        st->nc = pc;
-    }
 }
 
-__global__ void k_col_scatter(int n, const float4 *__restrict__ xw, const int *__restrict__ atom_col,
-                              const int *__restrict__ atom_slot,
-                              const int *__restrict__ col_atom_start,
-                              unsigned long long *__restrict__ keys) {
+// SCAN (ncol <= kScanInScatter): each block scans the columns itself, and
+// the first one writes the scans for the kernels that follow: one launch
+// less.
+template <bool SCAN>
+__global__ void __launch_bounds__(kScatterThreads) k_col_scatter(int n, int ncol, const float4 *__restrict__ xw,
+                                                                 const int *__restrict__ atom_col,
+                                                                 const int *__restrict__ atom_slot,
+                                                                 const int *__restrict__ col_count,
+                                                                 int *__restrict__ col_atom_start,
+                                                                 int *__restrict__ col_clus_start, nb_dev_state *st,
+                                                                 unsigned long long *__restrict__ keys) {
+    __shared__ int warp_a[32], warp_c[32], s_start[SCAN ? kScanInScatter + 1 : 1];
     nb_pdl_wait();
     nb_pdl_release();
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (SCAN) {
+        const bool over = scan_columns(ncol, col_count, warp_a, warp_c, [&](int c, int a, int k) {
+            s_start[c] = a;
+            if (blockIdx.x == 0) {
+                col_atom_start[c] = a;
+                col_clus_start[c] = k;
+                if (c == ncol) st->nc = k;
+            }
+        });
+        if (over && blockIdx.x == 0) atomicOr(&st->err, NB_DEV_COLUMN_OVERFLOW);
+        __syncthreads();
+    }
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     // z >= 0 after wrapping, so its bit pattern orders like the value
-    unsigned long long k = ((unsigned long long)__float_as_uint(xw[i].z) << 32) | (unsigned)i;
-    keys[col_atom_start[atom_col[i]] + atom_slot[i]] = k;
+    const unsigned long long k = ((unsigned long long)__float_as_uint(xw[i].z) << 32) | (unsigned)i;
+    const int col = atom_col[i];
+    keys[(SCAN ? s_start[col] : col_atom_start[col]) + atom_slot[i]] = k;
 }
 
 struct ColSortParams {
-    const int *col_count;
+    int *col_count;  // cleared for the next search
     const int *col_atom_start;
     const int *col_clus_start;
     const unsigned long long *keys;
@@ -179,6 +213,7 @@ struct ColSortParams {
 };
 
 constexpr int kSortWarps = 8;       // columns per CTA, one per warp
+constexpr int kFewColumns = 4;      // columns per SM up to which each has a CTA of its own
 constexpr int kWarpSortKeys = 256;  // a column up to this size is sorted in one warp's registers
 
 // Compare-exchange: a <= b afterwards if up, a >= b otherwise.
@@ -214,6 +249,11 @@ __device__ __forceinline__ void warp_bitonic_sort(unsigned long long (&v)[8], in
             }
         }
     }
+}
+
+// Atoms of a column that the sort takes (an overflow is flagged by the scan).
+__device__ __forceinline__ int column_atoms(const ColSortParams &p, int col) {
+    return min(p.col_atom_start[col + 1] - p.col_atom_start[col], NB_MAX_COL_ATOMS);
 }
 
 // The rest of a column once its cnt keys are sorted by z in sk: its z index,
@@ -290,7 +330,8 @@ __device__ __forceinline__ void finish_column(const ColSortParams &p, const unsi
 // at most kWarpSortKeys atoms is sorted by one warp in registers (no block
 // barriers) and a longer one, after those, by the whole CTA with a bitonic
 // sort in shared memory. The launch takes one column per CTA when columns
-// hold more than kWarpSortKeys / 2 atoms on average; the whole CTA then
+// hold more than kWarpSortKeys / 2 atoms on average, or when there are at
+// most kFewColumns of them per SM; the whole CTA then
 // sorts it (one warp alone was slower: its 36 dependent shuffle stages are
 // not shared out). Shared memory: NB_MAX_COL_ATOMS keys, kWarpSortKeys of
 // them per warp for short columns.
@@ -304,7 +345,8 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_col_sort(ColSortParams p) {
     const int warp_max = p.cpc > 1 ? kWarpSortKeys : 0;  // the longest column a warp sorts alone
     if (warp < p.cpc) {
         const int col = col0 + warp;
-        const int cnt = col < p.ncol ? min(p.col_count[col], NB_MAX_COL_ATOMS) : 0;
+        const int cnt = col < p.ncol ? column_atoms(p, col) : 0;
+        if (col < p.ncol && lane == 0) p.col_count[col] = 0;
         if (col < p.ncol && cnt <= warp_max) {
             const int a0 = p.col_atom_start[col];
             unsigned long long v[8];
@@ -324,7 +366,7 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_col_sort(ColSortParams p) {
     for (int w = 0; w < p.cpc; ++w) {  // the same decisions in every thread of the CTA
         const int col = col0 + w;
         if (col >= p.ncol) break;
-        const int cnt = min(p.col_count[col], NB_MAX_COL_ATOMS);  // overflow already flagged by the scan
+        const int cnt = column_atoms(p, col);
         if (cnt <= warp_max) continue;
         __syncthreads();  // every earlier use of sk is over
         const int a0 = p.col_atom_start[col];
@@ -360,18 +402,20 @@ cudaError_t nb_launch_grid_sort(nb_pairlist *pl, const float *coords, const nb_s
     nb_sys none;
     std::memset(&none, 0, sizeof(none));
     const int bs = 256, gb = (n + bs - 1) / bs;
-    const int gc = std::max(1, std::min((pl->ncol + bs - 1) / bs, 4 * pl->num_sms));
-    cudaError_t e = nb_launch_if(pdl, k_search_begin, gc, bs, 0, s, pl->sys, pl->sys_shift, one ? *one : none,
-                                  one ? 1 : 0, pl->col_count, pl->ncol, pl->st);
+    static_assert(kScatterThreads == 256, "the scatter's grid is k_bin's");
+    cudaError_t e = nb_launch_if(pdl, k_bin, gb, bs, 0, s, n, coords, (const int *)pl->atom_sys, pl->sys, pl->sys_shift,
+                                 one ? *one : none, one ? 1 : 0, pl->col_count, pl->atom_col, pl->atom_slot, pl->xw,
+                                 pl->st);
     if (e != cudaSuccess) return e;
-    e = nb_launch_if(pdl, k_bin, gb, bs, 0, s, n, coords, (const int *)pl->atom_sys, (const nb_sys *)pl->sys,
-                      pl->col_count, pl->atom_col, pl->atom_slot, pl->xw, pl->st);
-    if (e != cudaSuccess) return e;
-    e = nb_launch_if(pdl, k_col_scan, 1, 1024, 0, s, pl->ncol, (const int *)pl->col_count, pl->col_atom_start,
-                      pl->col_clus_start, pl->st);
-    if (e != cudaSuccess) return e;
-    e = nb_launch_if(pdl, k_col_scatter, gb, bs, 0, s, n, (const float4 *)pl->xw, (const int *)pl->atom_col,
-                      (const int *)pl->atom_slot, (const int *)pl->col_atom_start, pl->keys);
+    const bool scan_here = pl->ncol <= kScanInScatter;
+    if (!scan_here) {
+        e = nb_launch_if(pdl, k_col_scan, 1, 1024, 0, s, pl->ncol, (const int *)pl->col_count, pl->col_atom_start,
+                         pl->col_clus_start, pl->st);
+        if (e != cudaSuccess) return e;
+    }
+    e = nb_launch_if(pdl, scan_here ? k_col_scatter<true> : k_col_scatter<false>, gb, bs, 0, s, n, pl->ncol,
+                     (const float4 *)pl->xw, (const int *)pl->atom_col, (const int *)pl->atom_slot,
+                     (const int *)pl->col_count, pl->col_atom_start, pl->col_clus_start, pl->st, pl->keys);
     if (e != cudaSuccess) return e;
     ColSortParams cp;
     cp.col_count = pl->col_count;
@@ -391,6 +435,7 @@ cudaError_t nb_launch_grid_sort(nb_pairlist *pl, const float *coords, const nb_s
     cp.sys = pl->sys;
     cp.ztab = pl->ztab;
     cp.ncol = pl->ncol;
-    cp.cpc = (long long)n <= (long long)pl->ncol * (kWarpSortKeys / 2) ? kSortWarps : 1;
+    const bool many = pl->ncol > kFewColumns * pl->num_sms;
+    cp.cpc = many && (long long)n <= (long long)pl->ncol * (kWarpSortKeys / 2) ? kSortWarps : 1;
     return nb_launch_if(pdl, k_col_sort, (pl->ncol + cp.cpc - 1) / cp.cpc, kSortWarps * 32, 0, s, cp);
 }

@@ -157,9 +157,10 @@ extern "C" int nb_forces_noalloc(int n_atoms, const float *coords, const float *
 
     cudaStream_t s = (cudaStream_t)stream;
     // The scratch keeps the previous call's contents: reset the state block
-    // (error word, counters, cluster count) and the atom -> slot map, which
-    // the permute-back reads for every atom.
+    // (error word, counters, cluster count), the column counts and the atom ->
+    // slot map, which the permute-back reads for every atom.
     if (cudaMemsetAsync(pl.st, 0, sizeof(nb_dev_state), s) != cudaSuccess ||
+        cudaMemsetAsync(pl.col_count, 0, sizeof(int) * (size_t)pl.ncol, s) != cudaSuccess ||
         cudaMemsetAsync(pl.pos, 0, sizeof(int) * (size_t)n_atoms, s) != cudaSuccess ||
         cudaMemsetAsync(pl.atom_sys, 0, sizeof(int) * (size_t)n_atoms, s) != cudaSuccess ||
         cudaMemsetAsync(pl.col_sys, 0, sizeof(int) * (size_t)pl.ncol, s) != cudaSuccess)
