@@ -15,8 +15,8 @@
 //            (high word). i-forces stay in registers for the whole list of
 //            ci; j-forces are reduced across the four lanes sharing b with
 //            a reduce-scatter (3 shuffles) and added with one atomic per
-//            (atom, component) per 8x8 tile. Half-tiles (mask word 0) are
-//            skipped by a warp-uniform branch. Energies: per-lane FP32 per
+//            (atom, component) per 8x8 tile. Half-tiles with no pair in
+//            range are skipped by a warp-uniform branch. Energies: per-lane FP32 per
 //            tile, Kahan-compensated across tiles, FP64 per
 //            i-cluster and across the grid.
 // k_scatter  forces of cluster slots -> original atom order.
@@ -288,7 +288,6 @@ __global__ void __launch_bounds__(THREADS, 768 / THREADS) k_force(ForceParams p)
             for (int t = 0; t < nch; ++t) {
                 const int4 e = ent[t];
                 const float4 xj = sxj[t * NB_CLUSTER + b];
-                const int tj = stj[t * NB_CLUSTER + b];
                 const int sidx = e.y;
                 unsigned mlo = (unsigned)e.z, mhi = (unsigned)e.w;
                 if (p.part != NB_PART_ALL) {  // keep the pairs of this part: both atoms home, or not
@@ -298,21 +297,27 @@ __global__ void __launch_bounds__(THREADS, 768 / THREADS) k_force(ForceParams p)
                     mlo &= p.part == NB_PART_LOCAL ? l1 : ~l1;
                     mhi &= p.part == NB_PART_LOCAL ? l2 : ~l2;
                 }
+                // Which pairs are in range decides first: a half-tile without one is left out, and a
+                // tile without one leaves before its arithmetic, its reduction and its atomic
+                float4 S = make_float4(0.0f, 0.0f, 0.0f, 0.0f);  // adding S = 0 is exact
+                if (sidx != NB_SHIFT_CENTER) S = shift[sidx];
+                const float r1 = nb_r2(__fadd_rn(__fsub_rn(xi1.x, xj.x), S.x), __fadd_rn(__fsub_rn(xi1.y, xj.y), S.y),
+                                       __fadd_rn(__fsub_rn(xi1.z, xj.z), S.z));
+                const float r2 = nb_r2(__fadd_rn(__fsub_rn(xi2.x, xj.x), S.x), __fadd_rn(__fsub_rn(xi2.y, xj.y), S.y),
+                                       __fadd_rn(__fsub_rn(xi2.z, xj.z), S.z));
+                const bool in1 = (mlo & lanebit) != 0u && r1 < p.cc.rc2, in2 = (mhi & lanebit) != 0u && r2 < p.cc.rc2;
+                const bool any1 = __any_sync(0xffffffffu, in1), any2 = __any_sync(0xffffffffu, in2);
+                if (!(any1 || any2)) continue;
+                const int tj = stj[t * NB_CLUSTER + b];
                 float3 fj = make_float3(0.0f, 0.0f, 0.0f);
                 float ect = 0.0f, eljt = 0.0f;
                 int c1 = 0, c2 = 0;
-                if (sidx == NB_SHIFT_CENTER) {
-                    if (mlo) c1 = nb_pair<false, ENERGY, COUL>(xi1, qi1, xj, s_lj[tr1 + tj], 0.f, 0.f, 0.f,
-                                                         (mlo & lanebit) != 0u, p.cc, fi1, fj, ect, eljt);
-                    if (mhi) c2 = nb_pair<false, ENERGY, COUL>(xi2, qi2, xj, s_lj[tr2 + tj], 0.f, 0.f, 0.f,
-                                                         (mhi & lanebit) != 0u, p.cc, fi2, fj, ect, eljt);
-                } else {
-                    const float4 S = shift[sidx];
-                    if (mlo) c1 = nb_pair<true, ENERGY, COUL>(xi1, qi1, xj, s_lj[tr1 + tj], S.x, S.y, S.z,
-                                                        (mlo & lanebit) != 0u, p.cc, fi1, fj, ect, eljt);
-                    if (mhi) c2 = nb_pair<true, ENERGY, COUL>(xi2, qi2, xj, s_lj[tr2 + tj], S.x, S.y, S.z,
-                                                        (mhi & lanebit) != 0u, p.cc, fi2, fj, ect, eljt);
-                }
+                if (any1)
+                    c1 = nb_pair<true, ENERGY, COUL>(xi1, qi1, xj, s_lj[tr1 + tj], S.x, S.y, S.z, in1, p.cc, fi1, fj, ect,
+                                                     eljt);
+                if (any2)
+                    c2 = nb_pair<true, ENERGY, COUL>(xi2, qi2, xj, s_lj[tr2 + tj], S.x, S.y, S.z, in2, p.cc, fi2, fj, ect,
+                                                     eljt);
                 if (COUNT) cnt += c1 + c2;
                 // Reduce fj over the lanes l, l^8, l^16, l^24 (same b) as a
                 // reduce-scatter: afterwards lane l holds component comp.
