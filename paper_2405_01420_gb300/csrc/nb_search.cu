@@ -85,7 +85,17 @@ __device__ __forceinline__ int walk_candidates(const SearchParams &p, int ci, co
     const int jy0 = max((int)floorf((lo.y - p.rl_col) * S.inv_sy), -S.ncy);
     const int jy1 = min((int)floorf((hi.y + p.rl_col) * S.inv_sy), 2 * S.ncy - 1);
     const int nyr = jy1 - jy0 + 1;
-    const int ncols = (jx1 - jx0 + 1) * nyr;
+    // Clusters are numbered column by column, rows of columns (one jx) in order: rows before ci's hold
+    // no cluster cj >= ci. What is left of each image's rows, lx rows from ax on: about 28 columns
+    // away from the box's faces where the whole square has 49, so one batch in place of two.
+    const int cx = min(S.ncx - 1, max(0, (int)floorf(lo.x * S.inv_sx)));  // as the atom at lo.x was binned
+    int ax[3], lx[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        ax[k] = max(jx0, cx + (k - 1) * S.ncx);
+        lx[k] = max(min(jx1, k * S.ncx - 1) - ax[k] + 1, 0);
+    }
+    const int ncols = (lx[0] + lx[1] + lx[2]) * nyr;
     const float inv_nyr = 1.0f / (float)nyr;
     // cell edges; the binning's boundaries differ from these products by rounding only, far
     // below the 1e-3 nm by which rl_col exceeds the list radius
@@ -104,7 +114,10 @@ __device__ __forceinline__ int walk_candidates(const SearchParams &p, int ci, co
             int kxr = (int)((float)k * inv_nyr);
             kxr += (kxr + 1) * nyr <= k;
             kxr -= kxr * nyr > k;
-            const int jxu = jx0 + kxr, jyu = jy0 + (k - kxr * nyr);
+            const int jxu = kxr < lx[0] ? ax[0] + kxr
+                            : kxr < lx[0] + lx[1] ? ax[1] + (kxr - lx[0])
+                                                  : ax[2] + (kxr - lx[0] - lx[1]);
+            const int jyu = jy0 + (k - kxr * nyr);
             const int kx = image_of(jxu, S.ncx), ky = image_of(jyu, S.ncy);
             const int jx = jxu - kx * S.ncx, jy = jyu - ky * S.ncy;
             const int col = S.col_off + jx * S.ncy + jy;
