@@ -52,6 +52,8 @@
 
 namespace {
 
+constexpr unsigned kMaxPieces = 4u;  // pieces of a half's list in a small system
+
 struct VtParams {
     const float4 *xq;
     const int *tsort;
@@ -116,6 +118,16 @@ __device__ __forceinline__ VtJ load_j(const VtParams &p, int v, int t0, int t1, 
     return j;
 }
 
+// Pieces of each half's groups, one work item each (a small system without
+// energies, whose sums would depend on the split). 1,536 atoms, a call that
+// is waited for: 31.6 us with whole halves, 27.8 with up to 4 pieces.
+template <bool SPLIT>
+__device__ __forceinline__ unsigned vt_pieces(unsigned grid_warps, unsigned halves) {
+    return SPLIT ? min(nb_work_split(grid_warps, halves), kMaxPieces) : 1u;
+}
+
+__device__ __forceinline__ void prefetch_l1(const void *p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
+
 // The next work item: from the counter, past the items handed out by index.
 __device__ __forceinline__ unsigned take_item(const VtParams &p, unsigned by_index, int lane) {
     unsigned w = 0;
@@ -178,7 +190,8 @@ __global__ void __launch_bounds__(THREADS, RES) k_force_vt(VtParams p) {
     const unsigned nhalf = 2u * (unsigned)p.st->nc;  // halves per region
     const unsigned n0 = p.reg0 == 0 ? nhalf : 0u;
     const unsigned n1 = p.reg0 + p.nreg == 2 ? (p.nl_list ? p.st->nl_count : nhalf) : 0u;
-    const unsigned nwork = n0 + n1;
+    const unsigned nseg = vt_pieces<FIRST_BY_INDEX && !ENERGY>(gridDim.x * kWarps, n0 + n1);
+    const unsigned nwork = (n0 + n1) * nseg;
     if (ENERGY && lane == 0) s_e[warp][0] = s_e[warp][1] = 0.0;
     int cur_sys = -1;
     unsigned cnt = 0;
@@ -188,13 +201,14 @@ __global__ void __launch_bounds__(THREADS, RES) k_force_vt(VtParams p) {
     if (!FIRST_BY_INDEX) w = take_item(p, 0u, lane);
     for (;;) {
         unsigned reg = 0u, hw = 0u;
+        const unsigned u = nseg == 1u ? w : w / nseg, seg = w - u * nseg;
         int ci = 0;
-        if (w < n0) {
-            hw = w;
+        if (u < n0) {
+            hw = u;
             ci = (int)(hw >> 1);
         } else if (w < nwork) {
             reg = 1u;
-            hw = p.nl_list ? (unsigned)p.nl_list[w - n0] : w - n0;
+            hw = p.nl_list ? (unsigned)p.nl_list[u - n0] : u - n0;
             ci = (int)(hw >> 1);
         }
         const int h = (int)(hw & 1u);
@@ -205,7 +219,13 @@ __global__ void __launch_bounds__(THREADS, RES) k_force_vt(VtParams p) {
         }
         if (w >= nwork) break;
         const size_t hidx = (size_t)reg * p.reg_stride + 2 * ci + h;
-        const int t0 = p.half_start[hidx], t1 = t0 + p.half_len[hidx];
+        int t0 = p.half_start[hidx], t1 = t0 + p.half_len[hidx];
+        if (nseg > 1u) {
+            int g0, g1;
+            nb_piece((t1 - t0 + 3) >> 2, seg, nseg, g0, g1);
+            t1 = min(t1, t0 + 4 * g1);
+            t0 += 4 * g0;
+        }
         if (t1 <= t0) {
             w = take_item(p, by_index, lane);
             continue;
@@ -431,6 +451,7 @@ cudaError_t nb_launch_force_vt(nb_pairlist *pl, int ntype, const float *ljparams
     const int per_sm = occ.per_sm;
     const int use = pl->force_blocks_per_sm > 0 ? min(pl->force_blocks_per_sm, per_sm) : per_sm;
     int blocks = pl->num_sms * use;
-    blocks = min(blocks, (2 * p.nreg * pl->nc_max + threads / 32 - 1) / (threads / 32));
+    const long long items = 2LL * p.nreg * pl->nc_max * (shape == kShapeIndex && !e ? kMaxPieces : 1u);
+    blocks = (int)min((long long)blocks, (items + threads / 32 - 1) / (threads / 32));
     return nb_launch_pdl(fn, max(blocks, 1), threads, smem, s, p);
 }
