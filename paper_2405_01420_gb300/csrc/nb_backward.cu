@@ -206,6 +206,8 @@ __global__ void __launch_bounds__(kBwdThreads) k_backward(BwdParams p) {
 __global__ void k_bwd_scatter(int n, const int *__restrict__ pos, const float4 *__restrict__ bsort,
                               float *__restrict__ grad_x, float *__restrict__ grad_q, int ntype,
                               const double *__restrict__ acc, double *__restrict__ grad_lj) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int slot = i < n ? pos[i] : 0;  // the search's: before the wait
     nb_pdl_wait();
     nb_pdl_release();
     if (blockIdx.x == 0 && threadIdx.x < ntype * ntype) {
@@ -213,9 +215,8 @@ __global__ void k_bwd_scatter(int n, const int *__restrict__ pos, const float4 *
         grad_lj[2 * k] = 0.5 * (acc[2 * k] + acc[2 * kt]);
         grad_lj[2 * k + 1] = 0.5 * (acc[2 * k + 1] + acc[2 * kt + 1]);
     }
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const float4 v = bsort[pos[i]];
+    const float4 v = bsort[slot];
     grad_x[3 * i + 0] = v.x;
     grad_x[3 * i + 1] = v.y;
     grad_x[3 * i + 2] = v.z;

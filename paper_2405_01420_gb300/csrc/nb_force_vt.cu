@@ -160,6 +160,23 @@ __global__ void __launch_bounds__(THREADS, RES) k_force_vt(VtParams p) {
     __shared__ int s_tr[kWarps][4];
     __shared__ float4 s_xp[kWarps][2][2];  // row pair k: (x_a, x_b, y_a, y_b), (z_a, z_b, fq_a, fq_b)
     __shared__ double s_e[kWarps][2];      // the warp's energies of its current system: Coulomb, LJ
+    if (FIRST_BY_INDEX && p.nreg == 1 && p.reg0 == 0) {
+        // the warp's first tiles, which the prune wrote, on their way while the gather runs
+        const unsigned nh = 2u * (unsigned)p.st->nc, k = blockIdx.x * kWarps + (threadIdx.x >> 5);
+        const unsigned pieces = vt_pieces<FIRST_BY_INDEX && !ENERGY>(gridDim.x * kWarps, nh), u = k / pieces;
+        if (u < nh) {
+            int g0, g1;
+            const int len = p.half_len[u], lane = threadIdx.x & 31;
+            nb_piece((len + 3) >> 2, k - u * pieces, pieces, g0, g1);
+            const int tile = 4 * g0 + (lane >> 3);
+            if (tile < len) {
+                const size_t t = (size_t)p.half_start[u] + tile;
+                prefetch_l1(p.vt_slot + 8 * t + (lane & 7));
+                prefetch_l1(p.vt_mask + t);
+            }
+            prefetch_l1(p.clus_sys + (u >> 1));
+        }
+    }
     nb_pdl_wait();  // launched with nb_launch_pdl: the gather has completed from here on
     nb_pdl_release();
     const int nt2 = p.ntype * p.ntype;

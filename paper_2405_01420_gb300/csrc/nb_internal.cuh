@@ -206,8 +206,13 @@ __device__ __forceinline__ void nb_piece(int len, unsigned seg, unsigned nseg, i
 // blocks fill SMs that the predecessor's tail leaves idle, so the launch
 // latency between dependent kernels is hidden. Such a kernel starts with
 // nb_pdl_wait() (the predecessor has completed and its writes are visible;
-// nothing is read or written before it) and then nb_pdl_release(), which
+// nothing is written before it) and then nb_pdl_release(), which
 // lets its own successor be scheduled once all of its blocks have started.
+// Since every block releases only after its own wait, whatever ran before the
+// predecessor is complete when a block of the successor starts: before the
+// wait it may read what only such earlier kernels write, such as a search's
+// maps in a force call (never the caller's arrays, which the predecessor may
+// be writing).
 // Both are no-ops for a kernel launched the usual way.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void nb_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
