@@ -101,10 +101,11 @@ __device__ __forceinline__ void pme_offsets(const pme_axes &ax, const int base[3
     if (zc < 0) zc += ax.K[2];
 }
 
-// Clears the mesh ahead of the spread, which starts (with programmatic
-// dependent launch) while this runs. Launched the usual way, so everything
-// before it in the stream has completed by then.
+// Clears the mesh ahead of the spread, which starts (programmatic dependent
+// launch, as for all three kernels here) while this runs; everything before
+// this kernel in the stream has completed by then.
 __global__ void __launch_bounds__(kThreads) k_pme_clear(float *__restrict__ grid, unsigned cells) {
+    nb_pdl_wait();
     nb_pdl_release();
     const unsigned t = blockIdx.x * kThreads + threadIdx.x, stride = gridDim.x * kThreads;
     if (((size_t)grid & 15u) == 0) {
@@ -152,6 +153,7 @@ __global__ void __launch_bounds__(kThreads) k_pme_spread(int n, const float *__r
     pme_part r;
     if (i < (unsigned)n) r = pme_load(i, c, coords, q, ax);
     nb_pdl_wait();
+    nb_pdl_release();
     while (i < (unsigned)n) {
 #pragma unroll
         for (int a = 0; a < kOrder; ++a) {
@@ -172,6 +174,8 @@ __global__ void __launch_bounds__(kThreads) k_pme_gather(int n, const float *__r
                                                          const float *__restrict__ q, pme_axes ax,
                                                          const float *__restrict__ phi, float *__restrict__ forces,
                                                          int accumulate, double *__restrict__ energy) {
+    nb_pdl_wait();
+    nb_pdl_release();
     const int c = threadIdx.x & (kLanesPerAtom - 1);
     const int first = (threadIdx.x & 31) >> 2;  // the lane's atom among the warp's 8
     // unsigned: n < 2^31 and the stride is below 2^17, so i0 + stride never wraps
@@ -326,8 +330,7 @@ extern "C" int nb_pme_spread(int n_atoms, const float *coords, const float *q, c
     cudaStream_t s = (cudaStream_t)stream;
     const unsigned cells = (unsigned)((size_t)K0 * K1 * K2);
     constexpr unsigned per_block = 16 * kThreads;
-    k_pme_clear<<<(cells + per_block - 1) / per_block, kThreads, 0, s>>>(grid, cells);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = nb_launch_pdl(k_pme_clear, (int)((cells + per_block - 1) / per_block), kThreads, 0, s, grid, cells);
     if (e == cudaSuccess && n_atoms > 0)
         e = nb_launch_pdl(k_pme_spread, pme_blocks(n_atoms, (const void *)k_pme_spread, 0), kThreads, 0, s, n_atoms,
                           coords, q, ax, grid);
@@ -347,9 +350,8 @@ extern "C" int nb_pme_gather(int n_atoms, const float *coords, const float *q, c
     if (energy) e = cudaMemsetAsync(energy, 0, sizeof(double), s);
     if (e == cudaSuccess && n_atoms > 0) {
         const auto kernel = energy ? k_pme_gather<true> : k_pme_gather<false>;
-        kernel<<<pme_blocks(n_atoms, (const void *)kernel, energy ? 2 : 1), kThreads, 0, s>>>(
-            n_atoms, coords, q, ax, phi, forces, accumulate ? 1 : 0, energy);
-        e = cudaGetLastError();
+        e = nb_launch_pdl(kernel, pme_blocks(n_atoms, (const void *)kernel, energy ? 2 : 1), kThreads, 0, s, n_atoms, coords,
+                          q, ax, phi, forces, accumulate ? 1 : 0, energy);
     }
     if (e != cudaSuccess) return nb_record_error(NB_ERR_CUDA, cudaGetErrorString(e));
     return NB_OK;
