@@ -7,7 +7,8 @@ with few columns, one warp with many).
 
 Random points without exclusions: every pair within rlist by the FP32 distance
 contract has its mask bit exactly once, so the pair sets are compared bit for
-bit; there is no tolerance.
+bit; there is no tolerance. The same for the pruned list at positions moved
+since the search, whose clusters the prune first compares by their boxes.
 """
 import numpy as np
 import pytest
@@ -23,7 +24,7 @@ pytestmark = pytest.mark.gpu
 # columns per SM, by warp)
 BOXES = [((1.61, 1.61, 9.0), 700), ((9.0, 1.61, 1.61), 700), ((1.61, 9.0, 1.61), 700), ((1.61, 1.61, 1.61), 5),
          ((2.0, 3.1, 4.3), 333), ((5.0, 1.7, 1.7), 1500), ((6.3, 6.1, 1.62), 9001), ((40.0, 41.0, 1.61), 12007)]
-RLIST = 0.8
+RLIST, R_INNER = 0.8, 0.7
 
 
 def check(pl, nb, box, n, seed):
@@ -38,6 +39,14 @@ def check(pl, nb, box, n, seed):
     assert pl.status() == 0
     counted = expand_counted_pairs(pl.export(nb.NB_LIST_OUTER), oracle.image_f32(x, x, L), L, RLIST)
     ref = oracle.pairs_f32(x, x, L, RLIST, eo, ei)
+    assert len(pair_set(counted)) == len(counted)
+    assert pair_set(counted) == pair_set(ref)
+    # moved by at most 0.035 nm, less than half the margin of 0.1 nm between rlist and r_inner
+    moved = (x + rng.uniform(-0.02, 0.02, x.shape)).astype(np.float32)
+    pl.prune(torch.from_numpy(moved).cuda(), R_INNER)
+    assert pl.status() == 0
+    counted = expand_counted_pairs(pl.export(nb.NB_LIST_INNER), oracle.image_f32(x, moved, L), L, R_INNER)
+    ref = oracle.pairs_f32(x, moved, L, R_INNER, eo, ei)
     assert len(pair_set(counted)) == len(counted)
     assert pair_set(counted) == pair_set(ref)
 
