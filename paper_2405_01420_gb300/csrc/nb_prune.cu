@@ -1,7 +1,7 @@
 // Rolling prune (§III-A, "Prune-only kernel"): outer list at rlist ->
 // inner list at r_inner, with atom-pair in-range masks. As in the paper's
 // post-pruning list sorting, the prune also computes the list-size
-// histogram that the sort needs.
+// histogram where a sort will need it (nb_prune_sorts).
 //
 // One warp per i-cluster (work counter). The outer entries are taken 32 at
 // a time, one per lane; the warp first stages the 32 j clusters in shared

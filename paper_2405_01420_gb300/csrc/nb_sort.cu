@@ -4,10 +4,13 @@
 //
 // The force kernel hands out i-clusters from a work counter; taking them in
 // order of decreasing list length lets the longest lists start first, so the
-// persistent grid ends with short items and a short tail.
+// persistent grid ends with short items and a short tail. For the kernels
+// over 8x8 tiles only: those over gathered tiles take the halves in cluster
+// order, in which half lists run from long to short already.
 //
 // k_len_hist     histogram of the per-i-cluster list lengths (after a search;
-//                after a prune the prune kernel builds it, as in the paper)
+//                a prune whose list the 8x8 kernels will read builds it, as in
+//                the paper)
 // k_len_offsets  exclusive scan of the histogram from the longest length down
 // k_len_scatter  ci -> order[offset(len) + rank within its length]
 #include "nb_internal.cuh"
