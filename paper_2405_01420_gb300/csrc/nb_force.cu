@@ -72,8 +72,10 @@ struct GatherSlot {
 // ADJ: the gather of an adjoint call, which also brings dL/dF into cluster
 // order and clears the adjoint's accumulators in place of the forces'. One
 // kernel for both: a second one would read perm again and cost a launch.
+// 8 CTAs per SM (32 registers), the whole grid at once: at 6, with a slot's data loaded an iteration
+// ahead, a 256-box batch's gather took 86 us in place of 56.
 template <bool ADJ>
-__global__ void __launch_bounds__(256) k_gather(GatherParams p) {
+__global__ void __launch_bounds__(256, 8) k_gather(GatherParams p) {
     // What the search wrote may be read before the wait (nb_pdl_wait): a slot's atom, search
     // position and box are in flight while the kernel before this one ends (with the scatter's map and
     // the force kernel's first tiles: 894 -> 883 us per cycle of ten frames at 96,000 atoms)
@@ -85,10 +87,10 @@ __global__ void __launch_bounds__(256) k_gather(GatherParams p) {
     nb_pdl_wait();
     nb_pdl_release();
     float d2s_max = 0.0f, d2p_max = 0.0f;
-    for (; slot < nslot; slot += stride) {
+    for (bool first = true; slot < nslot; slot += stride, first = false) {
+        if (!first) next.load(p, slot);
         const int atom = next.atom;
         const float4 r = next.r, L = next.L;
-        if (slot + stride < nslot) next.load(p, slot + stride);
         if (ADJ) {
             p.bsort[slot] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             p.gsort[slot] = atom < 0 ? make_float4(0.0f, 0.0f, 0.0f, 0.0f)
