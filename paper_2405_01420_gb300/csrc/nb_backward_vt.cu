@@ -281,13 +281,17 @@ __global__ void __launch_bounds__(kBvtThreads, kBvtCtasPerSm) k_backward_vt(BvtP
         for (int k = 0; k < 2 * NT; ++k) acc[k][lane] = make_float4(0.f, 0.f, 0.f, 0.f);
         __syncwarp();
     }
-    // the CTA's LJ gradients, from its last warp
+    // The CTA's LJ gradients, from its last warp. Lane 0 hands over for its warp: the warp barriers order the
+    // other lanes' sums before its fence, and their reads of the other warps' sums after it (a shuffle orders
+    // no memory).
     unsigned done = 0u;
+    __syncwarp();
     if (lane == 0) {
         __threadfence_block();
         done = atomicAdd(&s_done, 1u);
         __threadfence_block();
     }
+    __syncwarp();
     if (__shfl_sync(0xffffffffu, done, 0) == kBvtWarps - 1 && lane < 2 * nt2) {
         double sum = 0.0;
 #pragma unroll
