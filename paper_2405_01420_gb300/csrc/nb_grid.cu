@@ -10,7 +10,9 @@
 //    of 8 into clusters, pads the last one, and writes the slot <-> atom
 //    maps, the search-frame positions and per-cluster bounding boxes. Clears
 //    the column counts, which are 0 between searches: a kernel of its own for
-//    that, at the start, cost a search of a small box 2 us.
+//    that, at the start, cost a search of a small box 2 us. Where a launch
+//    fails before it (a kernel loaded at its first use finds no memory, say),
+//    the counts are cleared with a memset there and then.
 //
 // Layout in HBM after the sort (slot = 8 * cluster + lane):
 //   perm[slot] (int), xref[slot] (float4), bbox[2c], bbox[2c+1] (float4).
@@ -397,9 +399,7 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_col_sort(ColSortParams p) {
     }
 }
 
-}  // namespace
-
-cudaError_t nb_launch_grid_sort(nb_pairlist *pl, const float *coords, const nb_sys *one, cudaStream_t s) {
+cudaError_t launch_kernels(nb_pairlist *pl, const float *coords, const nb_sys *one, cudaStream_t s) {
     const int n = pl->n_atoms;
     const bool pdl = pl->nc_max <= NB_SEARCH_PDL_MAX_CLUSTERS;
     nb_sys none;
@@ -441,4 +441,29 @@ cudaError_t nb_launch_grid_sort(nb_pairlist *pl, const float *coords, const nb_s
     const bool many = pl->ncol > kFewColumns * pl->num_sms;
     cp.cpc = many && (long long)n <= (long long)pl->ncol * (kWarpSortKeys / 2) ? kSortWarps : 1;
     return nb_launch_if(pdl, k_col_sort, (pl->ncol + cp.cpc - 1) / cp.cpc, kSortWarps * 32, 0, s, cp);
+}
+
+// Column counts of 0, for a sort that found or left others.
+cudaError_t clear_counts(nb_pairlist *pl, cudaStream_t s) {
+    const cudaError_t e = cudaMemsetAsync(pl->col_count, 0, sizeof(int) * (size_t)pl->ncol_max, s);
+    if (e == cudaSuccess) pl->col_dirty = 0;
+    return e;
+}
+
+}  // namespace
+
+// Counts left by a sort that failed would be added to by the next one, whose
+// keys would then be written past their end: they are cleared at the failure,
+// also for the sake of captured searches, and if that fails too, by the next
+// call.
+cudaError_t nb_launch_grid_sort(nb_pairlist *pl, const float *coords, const nb_sys *one, cudaStream_t s) {
+    cudaError_t e = pl->col_dirty ? clear_counts(pl, s) : cudaSuccess;
+    if (e != cudaSuccess) return e;
+    pl->col_dirty = 1;
+    e = launch_kernels(pl, coords, one, s);
+    if (e == cudaSuccess)
+        pl->col_dirty = 0;
+    else
+        clear_counts(pl, s);
+    return e;
 }

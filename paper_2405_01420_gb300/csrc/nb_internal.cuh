@@ -95,6 +95,7 @@ struct nb_pairlist {
     // device buffers
     nb_dev_state *st;
     int *col_count;       // [ncol_max] atoms per column during a grid sort, 0 between searches
+    int col_dirty;        // a grid sort did not get to the launch that clears them again
     int *col_atom_start;  // [ncol_max + 1]
     int *col_clus_start;  // [ncol_max + 1]
     int *atom_col;        // [N]
