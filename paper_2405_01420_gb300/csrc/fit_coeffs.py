@@ -80,35 +80,3 @@ if __name__ == "__main__":
     c = fit_exp2()
     print("EXP2:", ", ".join(f"{v:.9e}f" for v in c.astype(np.float32)))
 
-
-# --------------------------------------------------------------------------
-# H(x) = erfcx(x) + 2x/sqrt(pi) = P(x)/Q(x) on [0, X_MAX], degrees 4 and 3,
-# P(0) = Q(0) = 1: the Ewald pair force is q_a q_b exp(-x^2) H(x) / r^3 with
-# x = beta r. Same linearised fit, with weights raised where the error is
-# largest (Lawson) so that it levels out. Relative error 3.4e-8 in FP64,
-# 2.5e-7 evaluated in FP32 (erfcx above: 2.9e-7).
-# --------------------------------------------------------------------------
-def fit_h(n: int = 4, m: int = 3, x_max: float = X_MAX, rounds: int = 200):
-    t = 0.5 * (1.0 - np.cos(np.pi * (np.arange(20001) + 0.5) / 20001))
-    y = erfcx(x_max * t) + 2.0 / np.sqrt(np.pi) * x_max * t
-    vp, vq = np.vander(t, n + 1, increasing=True), np.vander(t, m + 1, increasing=True)
-    lw, qv, best = np.ones_like(t), np.ones_like(t), None
-    for _ in range(rounds):
-        for _ in range(6):
-            w = lw / (y * qv)
-            a = np.hstack([vp, -(y[:, None] * vq[:, 1:])]) * w[:, None]
-            c, *_ = np.linalg.lstsq(a, y * w, rcond=None)
-            q = np.concatenate([[1.0], c[n + 1:]])
-            qv = vq @ q
-        e = np.abs((vp @ c[: n + 1]) / qv / y - 1.0)
-        if best is None or e.max() < best[0]:
-            best = (e.max(), c[: n + 1] / x_max ** np.arange(n + 1), q / x_max ** np.arange(m + 1))
-        lw = lw * (e / e.max() + 0.02) ** 0.3
-        lw /= lw.max()
-    return best
-
-
-if __name__ == "__main__":
-    err, p, q = fit_h()
-    print("H P:", ", ".join(f"{v:.9e}" for v in p.astype(np.float32)))
-    print("H Q:", ", ".join(f"{v:.9e}" for v in q.astype(np.float32)), "max rel error:", err)

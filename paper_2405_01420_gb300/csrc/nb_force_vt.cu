@@ -35,8 +35,8 @@
 //  - Energies: FP32 over a half (per lane, then across the warp), FP64
 //    across halves in a per-warp shared pair (no registers held across
 //    halves), FP64 atomics per system when the warp moves to another
-//    system or finishes. Without energies the pair forces take fewer
-//    operations (nb_pair_x2: 797 -> 739 us at 1,000,002 atoms).
+//    system or finishes. The pair forces are the same bits with and without
+//    energies (nb_pair_x2).
 //  - Halves are handed out in cluster order. Half lists make the first
 //    clusters' lists the longest and the last ones' the shortest, so the
 //    launch ends with short items as it would in sorted order, and neither
@@ -44,8 +44,8 @@
 //    slower per call at 96,000 atoms, 4 us at 1,000,002).
 //  - First items (FIRST_BY_INDEX): from the work counter, or from the warp's index in
 //    the grid. The counter serves one warp per 1.3 ns, so 3,040 warps start
-//    over 4 us: a loss when each takes only a few halves (11,997 atoms: 22.0
-//    us per call from the counter, 18.1 from the index), a gain of 1 to 5%
+//    over 4 us: a loss when each takes only a few halves (12,000 atoms: 23.3
+//    us per call from the counter, 18.6 from the index), a gain of up to 6%
 //    when it takes many (the warps' phases are spread from the start).
 #include "nb_pair_x2.cuh"
 #include "nb_warp.cuh"
@@ -184,8 +184,7 @@ __global__ void __launch_bounds__(THREADS, RES) k_force_vt(VtParams p) {
     const int nt2 = p.ntype * p.ntype;
     for (int k = threadIdx.x; k < nt2; k += blockDim.x) {
         const float c6 = p.ljparams[2 * k], c12 = p.ljparams[2 * k + 1];
-        s_lj[k] = ENERGY ? make_float4(c6, c12, c12 * p.rc12inv - c6 * p.rc6inv, 0.0f)
-                         : make_float4(-6.0f * c6, nb_lj12_scale(COUL) * c12, 0.0f, 0.0f);
+        s_lj[k] = make_float4(c6, c12, c12 * p.rc12inv - c6 * p.rc6inv, 0.0f);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const unsigned ds = p.st->cur_d2_search, dp = p.st->cur_d2_prune;
@@ -386,25 +385,26 @@ using VtFn = void (*)(VtParams);
 // Launch shapes (threads, resident CTAs per SM, first items by index). The
 // default of 128 threads picks by the halves there are per warp of the grid;
 // microseconds per force call at 5 CTAs from the counter, then the shape
-// taken (rc 1.0, water):
+// taken (rc 1.0, water; replays of 20 or more calls without energies):
 //   without energies, up to 3.5 halves per warp: 5 CTAs by index
-//     (6,000 atoms 21.1 -> 15.5, 24,000 26.7 -> 26.0, 36,000 34.5 -> 34.2;
-//     48,000 42.2 -> 42.5, 96,000 80.8 -> 81.5)
-//   without energies, from 10 halves per warp: 6 CTAs (77 registers)
-//     (96,000 80.8 -> 81.0, 192,000 155 -> 152, 1,000,002 740 -> 712)
+//     (6,000 atoms 21.9 -> 15.7, 24,000 28.6 -> 27.6, 36,000 37.5 -> 37.5;
+//     96,000 84.4 -> 84.7, 1,000,002 825 -> 880; RF 12,000 17.4 -> 15.4)
+//   reaction field without energies, from 10 halves per warp: 6 CTAs (80
+//     registers; 96,000 59.9 -> 59.8, 192,000 128 -> 122). Ewald gains
+//     nothing by it (192,000 164 -> 166, 1,000,002 825 -> 827)
 //   with energies, up to 6 halves per warp of 4 CTAs: 4 CTAs by index
 //     (6,000 25.4 -> 17.2, 24,000 36.1 -> 34.2, 48,000 57.4 -> 55.5;
 //     96,000 102.3 -> 106.8)
 // Counting kernels and 256 threads have one shape.
 enum { kShape256, kShapeCounter, kShapeIndex, kShapeMany, kShapes };
 
-int pick_shape(bool energy, bool count, int threads, long long halves, int num_sms) {
+int pick_shape(bool energy, bool count, int threads, int coul, long long halves, int num_sms) {
     if (threads == 256) return kShape256;
     if (count) return kShapeCounter;
     const long long per_cta = 4LL * num_sms;  // warps of the grid per resident CTA
     if (energy) return halves <= 6 * 4 * per_cta ? kShapeIndex : kShapeCounter;
     if (2 * halves <= 7 * 5 * per_cta) return kShapeIndex;
-    return halves >= 10 * 5 * per_cta ? kShapeMany : kShapeCounter;
+    return coul == NB_COULK_RF && halves >= 10 * 5 * per_cta ? kShapeMany : kShapeCounter;
 }
 
 template <bool E, bool C, int K, bool B>
@@ -412,7 +412,7 @@ VtFn pick_vt_shape(int shape) {
     if (shape == kShape256) return k_force_vt<E, C, 256, 2, false, K, B>;
     if constexpr (!C) {
         if (shape == kShapeIndex) return k_force_vt<E, C, 128, E ? 4 : 5, true, K, B>;
-        if constexpr (!E)
+        if constexpr (!E && K == NB_COULK_RF)
             if (shape == kShapeMany) return k_force_vt<E, C, 128, 6, false, K, B>;
     }
     return k_force_vt<E, C, 128, 5, false, K, B>;
@@ -428,7 +428,8 @@ VtFn pick_vt_coul(int shape, bool batch) {
 template <bool E, bool C>
 VtFn pick_vt(int shape, int coul, bool batch) {
     if (coul == NB_COULK_RF) return pick_vt_coul<E, C, NB_COULK_RF>(shape, batch);
-    if (E && coul == NB_COULK_EWALD_SHIFT) return pick_vt_coul<E, C, NB_COULK_EWALD_SHIFT>(shape, batch);
+    if constexpr (E)
+        if (coul == NB_COULK_EWALD_SHIFT) return pick_vt_coul<E, C, NB_COULK_EWALD_SHIFT>(shape, batch);
     return pick_vt_coul<E, C, NB_COULK_EWALD>(shape, batch);  // the shift does not change forces
 }
 
@@ -474,7 +475,7 @@ cudaError_t nb_launch_force_vt(nb_pairlist *pl, int ntype, const float *ljparams
     const int threads = pl->force_threads == 256 ? 256 : 128;
     // halves of all systems: one cluster per 8 atoms and at most one more per column
     const long long halves = 2LL * (pl->n_atoms / NB_CLUSTER + pl->ncol);
-    const int shape = pick_shape(e, c, threads, halves, pl->num_sms);
+    const int shape = pick_shape(e, c, threads, coul, halves, pl->num_sms);
     const bool batch = e && pl->nsys > 1;
     VtFn fn = e ? (c ? pick_vt<true, true>(shape, coul, batch) : pick_vt<true, false>(shape, coul, batch))
                 : (c ? pick_vt<false, true>(shape, coul, batch) : pick_vt<false, false>(shape, coul, batch));

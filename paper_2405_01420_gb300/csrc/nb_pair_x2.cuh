@@ -22,20 +22,7 @@ struct nb_coul2 {
     float2 nsh;              // -erfc(beta rc)/rc
     float2 m2krf, krf, ncrf;  // -2 k_rf, k_rf, -c_rf
     float2 krf_lo, ncrf_lo;   // k_rf and -c_rf residuals
-    float2 hp1, hp2, hp3, hp4, nhq1, nhq2, nhq3;  // of H(beta r) = P(r)/Q(r): P's, and minus Q's, coefficients
 };
-
-// H(x) = erfcx(x) + 2x/sqrt(pi) = P(x)/Q(x) on [0, 3.2], P(0) = Q(0) = 1
-// (fit_coeffs.py; relative error 3.4e-8 in FP64, 2.5e-7 evaluated in FP32).
-// The Ewald force needs erfc(beta r)/r + (2 beta/sqrt(pi)) exp(-beta^2 r^2)
-// = exp(-beta^2 r^2) H(beta r)/r and nothing else of erfc.
-#define NB_H_P1 1.628190398
-#define NB_H_P2 1.973892808
-#define NB_H_P3 1.097177505
-#define NB_H_P4 2.501471043e-01
-#define NB_H_Q1 1.628193855
-#define NB_H_Q2 9.738355875e-01
-#define NB_H_Q3 2.215888798e-01
 
 inline nb_coul2 nb_pack_coul(const nb_coul &c) {
     nb_coul2 r;
@@ -48,15 +35,6 @@ inline nb_coul2 nb_pack_coul(const nb_coul &c) {
     r.ncrf = make_float2(-c.crf, -c.crf);
     r.krf_lo = make_float2(c.krf_lo, c.krf_lo);
     r.ncrf_lo = make_float2(-c.crf_lo, -c.crf_lo);
-    const double b = c.beta;  // the powers of beta go into the coefficients
-    const auto two = [](double v) { return make_float2((float)v, (float)v); };
-    r.hp1 = two(NB_H_P1 * b);
-    r.hp2 = two(NB_H_P2 * b * b);
-    r.hp3 = two(NB_H_P3 * b * b * b);
-    r.hp4 = two(NB_H_P4 * b * b * b * b);
-    r.nhq1 = two(-NB_H_Q1 * b);
-    r.nhq2 = two(-NB_H_Q2 * b * b);
-    r.nhq3 = two(-NB_H_Q3 * b * b * b);
     return r;
 }
 
@@ -94,40 +72,31 @@ __device__ __forceinline__ float2 nb_erfcx_x2(float2 x) {
     return __fmul2_rn(p, y);
 }
 
-// exp(-beta^2 r^2) and erfc(beta r)/r + (2 beta/sqrt(pi)) exp(-beta^2 r^2),
-// for forces (energies need erfc(beta r)/r alone): one rational in place of
-// erfcx's and the addition, and the hardware's exp2 (relative error 2^-22)
-// in place of the polynomial that keeps the energies' sums free of bias.
-__device__ __forceinline__ float2 nb_ewald_force_x2(const nb_coul2 &cc, const float2 r2, const float2 rinv,
-                                                    float2 &ex) {
-    const float2 t = __fmul2_rn(cc.kexp, r2), r = __fmul2_rn(r2, rinv);
-    ex = make_float2(nb_ex2(t.x), nb_ex2(t.y));
-    float2 p = __ffma2_rn(cc.hp4, r, cc.hp3);
-    p = __ffma2_rn(p, r, cc.hp2);
-    p = __ffma2_rn(p, r, cc.hp1);
-    p = __ffma2_rn(p, r, nb_f2(1.0f));
-    float2 nq = __ffma2_rn(cc.nhq3, r, cc.nhq2);
-    nq = __ffma2_rn(nq, r, cc.nhq1);
-    nq = __ffma2_rn(nq, r, nb_f2(-1.0f));  // -Q
-    float2 y = make_float2(nb_rcp(-nq.x), nb_rcp(-nq.y));
-    y = __ffma2_rn(y, __ffma2_rn(nq, y, nb_f2(1.0f)), y);
-    return __fmul2_rn(__fmul2_rn(p, y), __fmul2_rn(ex, rinv));
+// exp(-beta^2 r^2) in ex and erfc(beta r)/r in a, for forces and energies
+// alike. Forces need only c2b ex + a: the hardware's exp2 and one rational
+// for erfcx(x) + 2x/sqrt(pi) made calls without energies 9 to 15% faster
+// (11,997 atoms 19.0 -> 17.3 us, 96,000 84 -> 73, 1,000,002 827 -> 700), but
+// in FP32 that rational is off by up to 2.5e-7 where this form is by 1.3e-7,
+// the hardware's exp2 by 2^-22, and the forces' error against FP64 grew by
+// 1 to 5%.
+__device__ __forceinline__ void nb_ewald_x2(const nb_coul2 &cc, const float2 r2, const float2 rinv, float2 &ex,
+                                            float2 &a) {
+    const float2 r = __fmul2_rn(r2, rinv);
+    ex = nb_exp2_x2(__fmul2_rn(cc.kexp, r2));
+    a = __fmul2_rn(__fmul2_rn(ex, nb_erfcx_x2(__fmul2_rn(cc.beta, r))), rinv);
 }
 
-// Scale of C12 in the force-only LJ table: the reaction field's pair force
-// takes 12 C12, Ewald's C12 as it is.
-__host__ __device__ constexpr float nb_lj12_scale(int coul) { return coul == NB_COULK_RF ? 12.0f : 1.0f; }
-
 // Rows a, b (displacements d* = (y_a - y_b) + S, f q_i in qi) against j
-// (charge qj, both lanes equal). lj = (C6_a, C6_b, C12_a, C12_b), or without
-// ENERGY (-6 C6_a, -6 C6_b, k C12_a, k C12_b) with k = nb_lj12_scale(COUL);
-// nshlj = minus the LJ shifts of a and b. in_a, in_b: the list mask bits. Adds the rows' forces to fi*, the j force (positive sign,
-// summed over rows) to gj*, and with ENERGY the pair energies to ec, elj.
+// (charge qj, both lanes equal). lj = (C6_a, C6_b, C12_a, C12_b), nshlj =
+// minus the LJ shifts of a and b. in_a, in_b: the list mask bits. Adds the
+// rows' forces to fi*, the j force (positive sign, summed over rows) to gj*,
+// and with ENERGY the pair energies to ec, elj. The forces are the same bits
+// with and without ENERGY.
 // Returns the number of the two pairs within rc.
 template <bool ENERGY, int COUL>
 __device__ __forceinline__ int nb_pair_x2(const float2 dx, const float2 dy, const float2 dz, const float2 qi,
-                                          const float2 qj, const float4 lj, const float2 nshlj, const bool in_a, const bool in_b, const float rc2,
-                                          const nb_coul2 &cc, float2 &fix, float2 &fiy, float2 &fiz, float2 &gjx,
+                                          const float2 qj, const float4 lj, const float2 nshlj, const bool in_a,
+                                          const bool in_b, const float rc2, const nb_coul2 &cc, float2 &fix, float2 &fiy, float2 &fiz, float2 &gjx,
                                           float2 &gjy, float2 &gjz, float2 &ec, float2 &elj) {
     const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
     const bool ia = in_a && (r2.x < rc2);
@@ -137,35 +106,17 @@ __device__ __forceinline__ int nb_pair_x2(const float2 dx, const float2 dy, cons
     const float2 rinv = __ffma2_rn(__fmul2_rn(nb_f2(-0.5f), y0), nres, y0);
     const float2 rinv2 = __fmul2_rn(rinv, rinv);
     const float2 rinv6 = __fmul2_rn(__fmul2_rn(rinv2, rinv2), rinv2);
+    const float2 v6 = __fmul2_rn(make_float2(lj.x, lj.y), rinv6);
+    const float2 v12 = __fmul2_rn(__fmul2_rn(make_float2(lj.z, lj.w), rinv6), rinv6);
+    const float2 slj = __fmul2_rn(__ffma2_rn(nb_f2(12.0f), v12, __fmul2_rn(nb_f2(-6.0f), v6)), rinv2);
     const float2 qq = __fmul2_rn(qi, qj);
-    float2 s, a, v6, v12;
-    if (ENERGY) {
-        v6 = __fmul2_rn(make_float2(lj.x, lj.y), rinv6);
-        v12 = __fmul2_rn(__fmul2_rn(make_float2(lj.z, lj.w), rinv6), rinv6);
-        const float2 slj = __fmul2_rn(__ffma2_rn(nb_f2(12.0f), v12, __fmul2_rn(nb_f2(-6.0f), v6)), rinv2);
-        if (COUL == NB_COULK_RF) {
-            s = __ffma2_rn(qq, __ffma2_rn(rinv, rinv2, cc.m2krf), slj);
-        } else {
-            const float2 r = __fmul2_rn(r2, rinv);
-            const float2 ex = nb_exp2_x2(__fmul2_rn(cc.kexp, r2));
-            a = __fmul2_rn(__fmul2_rn(ex, nb_erfcx_x2(__fmul2_rn(cc.beta, r))), rinv);
-            s = __ffma2_rn(__fmul2_rn(qq, __ffma2_rn(cc.c2b, ex, a)), rinv2, slj);
-        }
+    float2 s, a;
+    if (COUL == NB_COULK_RF) {
+        s = __ffma2_rn(qq, __ffma2_rn(rinv, rinv2, cc.m2krf), slj);
     } else {
-        if (COUL == NB_COULK_RF) {
-            // no energies, so no v6 and v12 of their own: 12 C12/r^6 - 6 C6 in one FMA
-            const float2 w = __ffma2_rn(make_float2(lj.z, lj.w), rinv6, make_float2(lj.x, lj.y));
-            s = __ffma2_rn(qq, __ffma2_rn(rinv, rinv2, cc.m2krf), __fmul2_rn(w, __fmul2_rn(rinv6, rinv2)));
-        } else {
-            // the repulsion is rounded as with energies: what is derived from the forces of close
-            // pairs (the gradient of a force-matching loss) is the same with and without them
-            const float2 v12n = __fmul2_rn(__fmul2_rn(make_float2(lj.z, lj.w), rinv6), rinv6);
-            const float2 slj = __fmul2_rn(
-                __ffma2_rn(nb_f2(12.0f), v12n, __fmul2_rn(make_float2(lj.x, lj.y), rinv6)), rinv2);
-            float2 ex;
-            const float2 e = nb_ewald_force_x2(cc, r2, rinv, ex);
-            s = __ffma2_rn(__fmul2_rn(qq, e), rinv2, slj);
-        }
+        float2 ex;
+        nb_ewald_x2(cc, r2, rinv, ex, a);
+        s = __ffma2_rn(__fmul2_rn(qq, __ffma2_rn(cc.c2b, ex, a)), rinv2, slj);
     }
     s.x = ia ? s.x : 0.0f;
     s.y = ib ? s.y : 0.0f;
@@ -198,11 +149,10 @@ __device__ __forceinline__ int nb_pair_x2(const float2 dx, const float2 dy, cons
 
 // Rows a, b (.x, .y) of the adjoint pair nb_pair_adj<true, COUL> against
 // one j atom, on the packed instructions: each lane performs the scalar
-// form's operations in its order (negations exact), but for the Ewald terms,
-// which come from nb_ewald_force_x2 (the adjoint has no energies), so the
-// LJ gradients of a row are bit-equal to nb_pair_adj's. Inputs: the rows'
-// displacements d* = (y_a - y_b) + S, f q_i in qi_f and g in gi*; the j
-// atom's charge qj, f q_j in qj_f and negated g in ngj*; the rows' C6, C12
+// form's operations in its order (negations exact; the scalar form's own
+// products and sums may be contracted). Inputs: the rows' displacements
+// d* = (y_a - y_b) + S, f q_i in qi_f and g in gi*; the j atom's charge qj,
+// f q_j in qj_f and negated g in ngj*; the rows' C6, C12
 // against the j atom's type; the list mask bits in_a, in_b. Adds to the rows'
 // (dL/dx, dL/dq) in bi*; adds to vj* the vector v that the j atom's dL/dx
 // loses (subtract it once per j atom), and to bjq the j atom's dL/dq; d6,
@@ -233,8 +183,9 @@ __device__ __forceinline__ void nb_pair_adj_x2(const float2 dx, const float2 dy,
         Bc = __fadd2_rn(rinv3, cc.m2krf);  // 1/r^3 - 2 k_rf
         cpr = __fmul2_rn(__fmul2_rn(nb_f2(-3.0f), qq), rinv3);
     } else {
-        float2 ex;
-        Bc = __fmul2_rn(nb_ewald_force_x2(cc, r2, rinv, ex), rinv2);
+        float2 ex, a;
+        nb_ewald_x2(cc, r2, rinv, ex, a);
+        Bc = __fmul2_rn(__ffma2_rn(cc.c2b, ex, a), rinv2);
         cpr = __ffma2_rn(nb_f2(-3.0f), __fmul2_rn(qq, Bc), __fmul2_rn(__fmul2_rn(nk2, qq), ex));
     }
     const float2 s = __fadd2_rn(__fmul2_rn(qq, Bc), slj);
