@@ -83,10 +83,10 @@ typedef struct {
 /* nb_config.flags: count the in-range pairs in nb_forces (nb_stats.pairs_last);
    costs about one instruction per pair, so it is off unless asked for. */
 #define NB_FLAG_COUNT_PAIRS 0x1u
-/* nb_config.flags: do not sort i-clusters by list length after a search or
-   prune (§III-A: the post-pruning list sorting that shortens the tail of the
-   force kernel; on by default, and done where the kernels over 8x8 tiles,
-   which take the clusters in that order, will read the list). */
+/* nb_config.flags: do not sort i-clusters by list length after each search
+   and prune (§III-A: the post-pruning list sorting that shortens the tail
+   of the force kernel; on by default. The kernels over 8x8 tiles take the
+   clusters in that order). */
 #define NB_FLAG_NO_LIST_SORT 0x2u
 /* nb_config.flags: after a prune, compute forces (nb_forces) and the adjoint
    (nb_backward) over the 8x8 cluster-pair tiles of the inner list instead

@@ -350,21 +350,12 @@ extern "C" int nb_search(nb_pairlist *pl, const float *coords, const float *box,
     return ok();
 }
 
-// Orders the i-clusters of the current list by length if that is still due,
-// ahead of a kernel over the 8x8 tiles (those over gathered tiles take the
-// clusters as they are).
+// Orders the i-clusters of a search's list by length if that is still due.
 static cudaError_t sort_if_pending(nb_pairlist *pl, cudaStream_t s) {
     if (!pl->sort_pending) return cudaSuccess;
-    if (pl->has_inner) {
-        // NB_FLAG_CLUSTER_TILES set after the prune. During a capture the order would not exist
-        // until the graph runs, so the clusters are taken as they are
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        const cudaError_t e = cudaStreamIsCapturing(s, &cap);
-        if (e != cudaSuccess || cap != cudaStreamCaptureStatusNone) return e;
-    }
     pl->sort_pending = 0;
     if (pl->flags & NB_FLAG_NO_LIST_SORT) return cudaSuccess;
-    const cudaError_t e = nb_launch_sort_by_length(pl, pl->has_inner ? pl->ci_len_inner : pl->ci_len_outer, false, s);
+    const cudaError_t e = nb_launch_sort_by_length(pl, pl->ci_len_outer, false, s);
     if (e == cudaSuccess) pl->sorted = 1;
     return e;
 }
@@ -376,14 +367,14 @@ extern "C" int nb_prune(nb_pairlist *pl, const float *coords, float r_inner, voi
         return fail(NB_ERR_ARG, "nb_prune: r_inner = %g must be in (0, rlist = %g]", r_inner, pl->rlist);
     DeviceGuard g(pl->device);
     cudaStream_t s = (cudaStream_t)stream;
-    // the snapshot gather also clears the list-length histogram when the prune fills it
+    // the snapshot gather also clears the list-length histogram that the prune fills
     NB_CUDA(nb_launch_gather(pl, coords, nullptr, nullptr, 1, 1, nullptr, NB_PART_ALL, s));
     const float r2cut = r_inner * r_inner;
+    const bool sort = !(pl->flags & NB_FLAG_NO_LIST_SORT);
     NB_CUDA(nb_launch_prune(pl, r2cut, stale_bound2(pl->rlist, r_inner), s));
     pl->sorted = 0;
-    pl->sort_pending = !(pl->flags & NB_FLAG_NO_LIST_SORT);
-    if (nb_prune_sorts(pl)) {
-        pl->sort_pending = 0;
+    pl->sort_pending = 0;
+    if (sort) {
         NB_CUDA(nb_launch_sort_by_length(pl, pl->len_key, true, s));
         pl->sorted = 1;
     }
@@ -421,12 +412,11 @@ static int forces_impl(const char *who, nb_pairlist *pl, int part, const float *
     const int kpart = split ? part : NB_PART_ALL;
     const bool last = part != NB_PART_LOCAL;  // this call ends the evaluation
     if (compute) {
-        const bool gathered = pl->has_vtiles && !(pl->flags & NB_FLAG_CLUSTER_TILES);
-        if (!gathered) NB_CUDA(sort_if_pending(pl, s));
+        NB_CUDA(sort_if_pending(pl, s));
         NB_CUDA(nb_launch_gather(pl, coords, q, type, ntype, 0, energies, kpart, s));
         if (pl->ev_start) NB_CUDA(cudaEventRecord(pl->ev_start, s));
         const int fpart = (!split && part == NB_PART_LOCAL) ? NB_PART_ALL : kpart;
-        if (gathered)
+        if (pl->has_vtiles && !(pl->flags & NB_FLAG_CLUSTER_TILES))
             NB_CUDA(nb_launch_force_vt(pl, ntype, ljparams, rc, beta, energies, stale_bound2(pl->r_inner, rc), fpart,
                                        s));
         else
@@ -472,7 +462,7 @@ extern "C" int nb_backward(nb_pairlist *pl, const float *coords, const float *q,
         return fail(NB_ERR_STATE, "nb_backward: NB_COUL_EXCL_CORR needs a search with exclusion lists made while it was set");
     DeviceGuard gd(pl->device);
     cudaStream_t s = (cudaStream_t)stream;
-    if (!pl->has_vtiles || (pl->flags & NB_FLAG_CLUSTER_TILES)) NB_CUDA(sort_if_pending(pl, s));
+    NB_CUDA(sort_if_pending(pl, s));
     NB_CUDA(nb_launch_gather_adj(pl, coords, q, type, ntype, g, s));
     NB_CUDA(nb_launch_backward(pl, ntype, ljparams, rc, beta, grad_x, grad_q, grad_lj, stale_bound2(pl->rlist, rc),
                                stale_bound2(pl->r_inner, rc), s));

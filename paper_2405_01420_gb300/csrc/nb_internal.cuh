@@ -133,7 +133,8 @@ struct nb_pairlist {
     int *ci_order;        // [nc_max] i-clusters by decreasing list length
     int sorted;           // an order was launched for the current list; whether ci_order still holds one for its
                           // clusters is known on the device (nb_order_valid)
-    int sort_pending;     // the current list is sorted by length at its first use by a kernel over 8x8 tiles
+    int sort_pending;     // the last search's list is sorted by length at its first use (unless a prune
+                          // comes first and sorts its own)
     int *vt_slot;         // [2 cap * 8] gathered tiles: j slot | shift << 27
     unsigned *vt_mask;    // [2 cap] 4 x 8 in-range bits per gathered tile
     int *half_start;      // [2 parts][2 nc_max] first gathered tile of each half i-cluster
@@ -279,12 +280,6 @@ cudaError_t nb_launch_prune(nb_pairlist *pl, float r_inner2, float stale_search2
 // Orders i-clusters by decreasing ci_len. hist_ready: the histogram of
 // ci_len is already in len_hist (the prune computes it), else it is built here.
 cudaError_t nb_launch_sort_by_length(nb_pairlist *pl, const int *ci_len, bool hist_ready, cudaStream_t s);
-// Whether a prune orders the i-clusters of its list: only the kernels over 8x8 tiles take them in
-// that order (histogram, offsets and order: 7 us of an 84 us prune call at 96,000 atoms). With
-// NB_FLAG_CLUSTER_TILES set later on, the first call that needs the order makes it.
-inline bool nb_prune_sorts(const nb_pairlist *pl) {
-    return !(pl->flags & NB_FLAG_NO_LIST_SORT) && (!pl->vt_slot || (pl->flags & NB_FLAG_CLUSTER_TILES));
-}
 // Clears the list-length histogram ahead of a prune that fills it.
 cudaError_t nb_clear_len_hist(nb_pairlist *pl, cudaStream_t s);
 // Records the excluded pairs of the caller's exclusion lists as slot pairs

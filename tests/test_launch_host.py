@@ -1,6 +1,7 @@
 """Launch logic of the library on the host, over a stand-in CUDA runtime:
 a pair search one of whose launches fails leaves nothing behind that the next
-one would take for its own."""
+one would take for its own; a prune orders its list whichever kernels are to
+read it."""
 import ctypes
 
 import numpy as np
@@ -69,4 +70,35 @@ def test_a_failed_search_leaves_no_counts(lib, kernel, memset_fails_too):
         assert search(lib, pl, (3, 4, 5)) == NB_OK
     assert len(rec.memsets) == n_memsets, "one clear is enough"
     assert counts.at_bin == [0] * len(counts.at_bin)
+    lib.nb_pairlist_destroy(pl)
+
+
+@pytest.mark.parametrize("capturing", [False, True])
+@pytest.mark.parametrize("sort_lists", [True, False])
+def test_cluster_tiles_turned_on_after_a_prune_find_an_order(lib, sort_lists, capturing):
+    from paper_2405_01420_gb300 import nb
+    pl = create(lib)
+    orders = []
+
+    def emulate(name, args):
+        if "k_forceI" in name:  # the parameter struct's seventh pointer
+            orders.append(ctypes.cast(args[0], ctypes.POINTER(ctypes.c_void_p))[6])
+
+    rec = fake_cuda.Recorder(lib, emulate)
+    assert lib.nb_set_flags(pl, 0 if sort_lists else nb.NB_FLAG_NO_LIST_SORT) == NB_OK
+    assert search(lib, pl, (3, 3, 3)) == NB_OK
+    x, q, t = np.zeros((N, 3), np.float32), np.zeros(N, np.float32), np.zeros(N, np.int32)
+    lj, F = np.zeros((1, 1, 2), np.float32), np.zeros((N, 3), np.float32)
+    assert lib.nb_prune(pl, x.ctypes.data, 0.7, None) == NB_OK
+    assert any("k_len_scatter" in k for k in rec.names) == sort_lists
+    rec.names.clear()
+    lib.fake_capturing(capturing)
+    flags = nb.NB_FLAG_CLUSTER_TILES | (0 if sort_lists else nb.NB_FLAG_NO_LIST_SORT)
+    assert lib.nb_set_flags(pl, flags) == NB_OK
+    for _ in range(2):
+        assert lib.nb_forces(pl, x.ctypes.data, q.ctypes.data, t.ctypes.data, 1, lj.ctypes.data, 0.6, 3.0,
+                             F.ctypes.data, None, None) == NB_OK
+    lib.fake_capturing(False)
+    assert len(orders) == 2 and all((o is not None) == sort_lists for o in orders)
+    assert not any("k_len" in k for k in rec.names), "the order is the prune's"
     lib.nb_pairlist_destroy(pl)
