@@ -150,13 +150,17 @@ def _check(code: int):
 def _stream(stream):
     """The stream's raw handle; None is the current device's current stream.
 
-    A small call's time is what the host takes to issue it (15 us for a force
-    call at 1,536 atoms), so neither this nor ``_dev`` builds an object where a
-    number will do: ctypes converts it by the declared argument type.
+    A small call's time is what the host takes to issue it (a force call at
+    1,536 atoms: 16 us with a Stream and a c_void_p for each argument, 10.7
+    so), so neither this nor ``_dev`` builds an object where a number will do:
+    ctypes converts it by the declared argument type.
     """
     if stream is None:
         if torch.cuda.is_initialized():
-            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+            try:  # not public: a torch without them takes the way below
+                return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+            except AttributeError:
+                pass
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream
