@@ -166,6 +166,7 @@ int alloc_pairlist(nb_pairlist *pl, long long n, const nb_config *cfg, const cha
     NB_CUDA(cudaMemset(pl->pos, 0, sizeof(int) * (size_t)n));
     NB_CUDA(cudaMemset(pl->perm, 0xff, sizeof(int) * nslot));
     NB_CUDA(cudaMemset(pl->ci_start, 0, sizeof(int) * (size_t)pl->nc_max));
+    NB_CUDA(cudaMemset(pl->ci_order, 0, sizeof(int) * (size_t)pl->nc_max));
     NB_CUDA(cudaMemset(pl->ci_len_outer, 0, sizeof(int) * (size_t)pl->nc_max));
     NB_CUDA(cudaMemset(pl->ci_len_inner, 0, sizeof(int) * (size_t)pl->nc_max));
     NB_CUDA(cudaMemset(pl->fsort, 0, sizeof(float4) * nslot));
@@ -316,6 +317,7 @@ extern "C" int nb_search(nb_pairlist *pl, const float *coords, const float *box,
         pl->ncol = ncx * ncy;
         pl->sys_host[0] = make_sys(box, ncx, ncy, 0, 0, pl->n_atoms);
     }
+    pl->sorted = 0;  // whatever becomes of this search, an order of earlier clusters is not for its own
     // the grid sort's first kernel clears the list counter and writes a single system's table
     NB_CUDA(nb_launch_grid_sort(pl, coords, pl->batch ? nullptr : &pl->sys_host[0], s));
 
@@ -337,7 +339,6 @@ extern "C" int nb_search(nb_pairlist *pl, const float *coords, const float *box,
     }
     // ordering the clusters by list length waits for the first force or adjoint call on this list: a
     // prune that comes first orders them by its own (pruned) work instead
-    pl->sorted = 0;
     // A system small enough that the force kernel splits every list four ways or more has no
     // launch tail for the ordering to shorten: its three kernels would only add latency.
     const bool small = (long long)pl->nc_max * 4 <= (long long)pl->num_sms * 32;

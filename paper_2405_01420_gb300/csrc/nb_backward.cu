@@ -95,14 +95,13 @@ __global__ void __launch_bounds__(kBwdThreads) k_backward(BwdParams p) {
     float4 *sgj = s_gj[warp];
     int *stj = s_tj[warp];
     const int nc = p.st->nc;
-    const bool ordered = nb_order_valid(p.order, p.st);
 
     for (;;) {
         unsigned w = 0;
         if (lane == 0) w = atomicAdd(&p.st->work, 1u);
         w = __shfl_sync(0xffffffffu, w, 0);
         if (w >= (unsigned)nc) break;
-        const int ci = ordered ? p.order[w] : (int)w;
+        const int ci = p.order ? p.order[w] : (int)w;
         const float4 *shift = p.sys_shift + 27 * p.clus_sys[ci];
         const int k0 = p.ci_start[ci], k1 = k0 + p.ci_len[ci];
         const float4 xi1 = p.xq[ci * NB_CLUSTER + a1], xi2 = p.xq[ci * NB_CLUSTER + a2];

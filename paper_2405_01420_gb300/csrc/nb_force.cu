@@ -173,7 +173,7 @@ struct ForceParams {
     const int4 *list;
     const int *ci_start;
     const int *ci_len;
-    const int *order;         // i-clusters by decreasing list length (used if nb_order_valid), or NULL
+    const int *order;         // i-clusters by decreasing list length, or NULL
     const float *ljparams;
     nb_dev_state *st;
     double *energies;         // [2 nsys]
@@ -246,7 +246,6 @@ __global__ void __launch_bounds__(THREADS, 768 / THREADS) k_force(ForceParams p)
     float4 *sxj = s_xj[warp];
     int *stj = s_tj[warp];
     const int nc = p.st->nc;
-    const bool ordered = nb_order_valid(p.order, p.st);
     double ecd = 0.0, eljd = 0.0;  // energies of system cur_sys not yet added to the output
     int cur_sys = -1;
     unsigned cnt = 0;
@@ -265,7 +264,7 @@ __global__ void __launch_bounds__(THREADS, 768 / THREADS) k_force(ForceParams p)
         }
         // work item w: range seg of the list of the i-cluster at position idx of the order
         const unsigned idx = nseg == 1u ? w : w / nseg, seg = w - idx * nseg;
-        const int ci = (w < nwork && ordered) ? p.order[idx] : (int)idx;
+        const int ci = (w < nwork && p.order) ? p.order[idx] : (int)idx;
         const int csys = (w < nwork) ? p.clus_sys[ci] : -1;
         if (ENERGY && csys != cur_sys) {
             if (cur_sys >= 0) flush_energies(ecd, eljd, lane, p.energies + 2 * cur_sys);

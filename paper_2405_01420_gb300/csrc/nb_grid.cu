@@ -37,10 +37,7 @@ __global__ void k_bin(int n, const float *__restrict__ coords, const int *__rest
     nb_pdl_release();
     if (blockIdx.x == 0) {
         const int k = threadIdx.x;
-        if (k == 0) {
-            st->list_count = 0ull;
-            st->searches += 1u;  // an order of earlier clusters no longer holds
-        }
+        if (k == 0) st->list_count = 0ull;
         if (single && k == 0) sys[0] = one;
         if (single && k < 27)
             sys_shift[k] = make_float4((float)nb_shift_x(k) * one.box.x, (float)nb_shift_y(k) * one.box.y,

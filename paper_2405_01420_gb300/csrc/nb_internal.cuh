@@ -36,10 +36,8 @@ struct nb_dev_state {
     unsigned cur_d2_prune;
     unsigned long long npairs;     // in-range pairs counted by the last force call
     unsigned excl_count;           // excluded pairs recorded by the last search
-    unsigned searches;             // searches run on this list so far, replays of captured ones included
     unsigned long long tile_count; // gathered tiles written by the last prune
     unsigned nl_count;             // halves with non-local tiles listed by the last prune (halo split)
-    unsigned order_search;         // `searches` when ci_order was made (see nb_order_valid)
 };
 
 // Per-system parameters (one entry per independent box). A single-system
@@ -54,17 +52,6 @@ struct nb_sys {
     int n_atoms;       // atoms of this system
     int pad;
 };
-
-// Whether ci_order is a permutation of the clusters there are now. The host
-// cannot know: a captured search makes new clusters, as many as its frame
-// needs, without a call of this library, and a captured force call keeps the
-// order's address over searches that make no new order. A kernel that is
-// given an order takes the clusters as they are where this does not hold. (An
-// order of another list over the same clusters, an unpruned one say, is a
-// permutation all the same.)
-__device__ __forceinline__ bool nb_order_valid(const int *order, const nb_dev_state *st) {
-    return order != nullptr && st->order_search == st->searches;
-}
 
 // Host handle. Device buffers are sized at creation for n_atoms.
 struct nb_pairlist {
@@ -130,9 +117,11 @@ struct nb_pairlist {
     int *len_key;         // [nc_max] per-i-cluster work after a prune (gathered tiles, else inner entries)
     int *len_offsets;     // [NB_LEN_BINS]
     int *len_cursor;      // [NB_LEN_BINS]
-    int *ci_order;        // [nc_max] i-clusters by decreasing list length
-    int sorted;           // an order was launched for the current list; whether ci_order still holds one for its
-                          // clusters is known on the device (nb_order_valid)
+    int *ci_order;        // [nc_max] the i-clusters, each once: by decreasing list length once they are ordered,
+                          // as they come (written by every search) before that. Always a permutation of the
+                          // clusters there are: captured searches make new ones, as many as their frame needs,
+                          // without a call of the library, and captured force calls keep this address
+    int sorted;           // an order by length was launched for the current list
     int sort_pending;     // the last search's list is sorted by length at its first use (unless a prune
                           // comes first and sorts its own)
     int *vt_slot;         // [2 cap * 8] gathered tiles: j slot | shift << 27

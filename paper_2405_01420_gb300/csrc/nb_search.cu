@@ -33,6 +33,7 @@ struct SearchParams {
     int4 *outer;
     int *ci_start;
     int *ci_len;
+    int *order;         // ci_order, or NULL
     int *ci_len_inner;
     nb_dev_state *st;
     const nb_sys *sys;
@@ -343,6 +344,7 @@ __global__ void __launch_bounds__(kSearchWarps * 32, 4) k_search(SearchParams p)
             p.ci_start[ci] = (int)base;
             p.ci_len[ci] = nkept;
             p.ci_len_inner[ci] = 0;
+            if (p.order) p.order[ci] = ci;  // an order of earlier clusters no longer holds
         }
         __syncwarp();
     }
@@ -364,6 +366,7 @@ cudaError_t nb_launch_search(nb_pairlist *pl, const int *excl_off, const int *ex
     p.ci_start = pl->ci_start;
     p.ci_len = pl->ci_len_outer;
     p.ci_len_inner = pl->ci_len_inner;
+    p.order = pl->ci_order;
     p.st = pl->st;
     p.sys = pl->sys;
     p.clus_sys = pl->clus_sys;

@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(NB_LEN_BINS) k_len_offsets(const int *__restri
 // Each pass of a CTA places kSortThreads clusters: ranks within the CTA by
 // shared atomics, then one global atomic per occupied bin reserves the
 // CTA's places in that bin.
-__global__ void __launch_bounds__(kSortThreads) k_len_scatter(const int *__restrict__ ci_len, nb_dev_state *st,
+__global__ void __launch_bounds__(kSortThreads) k_len_scatter(const int *__restrict__ ci_len, const nb_dev_state *st,
                                                               const int *__restrict__ offsets,
                                                               int *__restrict__ cursor, int *__restrict__ order) {
     __shared__ int s_cnt[NB_LEN_BINS];
@@ -68,7 +68,6 @@ __global__ void __launch_bounds__(kSortThreads) k_len_scatter(const int *__restr
     nb_pdl_wait();
     nb_pdl_release();
     const int nc = st->nc;
-    if (blockIdx.x == 0 && threadIdx.x == 0) st->order_search = st->searches;
     for (int c0 = blockIdx.x * blockDim.x; c0 < nc; c0 += gridDim.x * blockDim.x) {
         for (int b = threadIdx.x; b < NB_LEN_BINS; b += blockDim.x) s_cnt[b] = 0;
         __syncthreads();
@@ -100,6 +99,6 @@ cudaError_t nb_launch_sort_by_length(nb_pairlist *pl, const int *ci_len, bool hi
     cudaError_t e = nb_launch_pdl(k_len_offsets, 1, NB_LEN_BINS, 0, s, (const int *)pl->len_hist, pl->len_offsets,
                                   pl->len_cursor);
     if (e != cudaSuccess) return e;
-    return nb_launch_pdl(k_len_scatter, blocks, kSortThreads, 0, s, ci_len, pl->st,
+    return nb_launch_pdl(k_len_scatter, blocks, kSortThreads, 0, s, ci_len, (const nb_dev_state *)pl->st,
                          (const int *)pl->len_offsets, pl->len_cursor, pl->ci_order);
 }
