@@ -85,8 +85,8 @@ typedef struct {
 #define NB_FLAG_COUNT_PAIRS 0x1u
 /* nb_config.flags: do not sort i-clusters by list length after each search
    and prune (§III-A: the post-pruning list sorting that shortens the tail
-   of the force kernel; on by default. The kernels over 8x8 tiles take the
-   clusters in that order). */
+   of the force kernel; on by default, and done where the kernels over 8x8
+   tiles, which take the clusters in that order, will read the list). */
 #define NB_FLAG_NO_LIST_SORT 0x2u
 /* nb_config.flags: after a prune, compute forces (nb_forces) and the adjoint
    (nb_backward) over the 8x8 cluster-pair tiles of the inner list instead
@@ -309,8 +309,11 @@ int nb_set_timing_events(nb_pairlist *pl, void *start, void *stop);
  * Replace the pair list's NB_FLAG_* flags (set at creation through
  * nb_config.flags). Each flag takes effect at the next call that reads it:
  * NB_FLAG_COUNT_PAIRS and NB_FLAG_CLUSTER_TILES at nb_forces / nb_backward,
- * NB_FLAG_NO_LIST_SORT at nb_search / nb_prune. Used by the autotuner to
- * choose the tile form. Errors: NB_ERR_ARG for an unknown flag.
+ * NB_FLAG_NO_LIST_SORT at nb_search / nb_prune. A prune made while
+ * NB_FLAG_CLUSTER_TILES is set also orders its list by length; with the flag
+ * set after it, the first nb_forces / nb_backward call over it does (each
+ * such call that is captured, or that follows a captured prune). Used by the
+ * autotuner to choose the tile form. Errors: NB_ERR_ARG for an unknown flag.
  */
 int nb_set_flags(nb_pairlist *pl, unsigned flags);
 

@@ -351,12 +351,33 @@ extern "C" int nb_search(nb_pairlist *pl, const float *coords, const float *box,
     return ok();
 }
 
-// Orders the i-clusters of a search's list by length if that is still due.
+static cudaError_t is_capturing(cudaStream_t s, bool &yes) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(s, &status);
+    yes = status != cudaStreamCaptureStatusNone;
+    return e;
+}
+
+// Orders the i-clusters of the current list by length if that is still due,
+// ahead of a kernel over the 8x8 tiles (those over gathered tiles take the
+// clusters as they are).
 static cudaError_t sort_if_pending(nb_pairlist *pl, cudaStream_t s) {
     if (!pl->sort_pending) return cudaSuccess;
-    pl->sort_pending = 0;
-    if (pl->flags & NB_FLAG_NO_LIST_SORT) return cudaSuccess;
-    const cudaError_t e = nb_launch_sort_by_length(pl, pl->ci_len_outer, false, s);
+    bool once = true;
+    if (pl->has_inner) {
+        // NB_FLAG_CLUSTER_TILES set after the prune. An order made in a capture exists only when its graph
+        // runs, and a captured prune makes further lists: then each call makes its own (6 us)
+        bool capturing = false;
+        const cudaError_t e = is_capturing(s, capturing);
+        if (e != cudaSuccess) return e;
+        once = !capturing && !pl->prune_captured;
+    }
+    if (once) pl->sort_pending = 0;
+    if (pl->flags & NB_FLAG_NO_LIST_SORT) {
+        pl->sorted = 0;
+        return cudaSuccess;
+    }
+    const cudaError_t e = nb_launch_sort_by_length(pl, pl->has_inner ? pl->ci_len_inner : pl->ci_len_outer, false, s);
     if (e == cudaSuccess) pl->sorted = 1;
     return e;
 }
@@ -368,14 +389,17 @@ extern "C" int nb_prune(nb_pairlist *pl, const float *coords, float r_inner, voi
         return fail(NB_ERR_ARG, "nb_prune: r_inner = %g must be in (0, rlist = %g]", r_inner, pl->rlist);
     DeviceGuard g(pl->device);
     cudaStream_t s = (cudaStream_t)stream;
-    // the snapshot gather also clears the list-length histogram that the prune fills
+    bool capturing = false;
+    NB_CUDA(is_capturing(s, capturing));
+    // the snapshot gather also clears the list-length histogram when the prune fills it
     NB_CUDA(nb_launch_gather(pl, coords, nullptr, nullptr, 1, 1, nullptr, NB_PART_ALL, s));
     const float r2cut = r_inner * r_inner;
-    const bool sort = !(pl->flags & NB_FLAG_NO_LIST_SORT);
     NB_CUDA(nb_launch_prune(pl, r2cut, stale_bound2(pl->rlist, r_inner), s));
     pl->sorted = 0;
-    pl->sort_pending = 0;
-    if (sort) {
+    pl->sort_pending = !(pl->flags & NB_FLAG_NO_LIST_SORT);
+    pl->prune_captured = capturing;
+    if (nb_prune_sorts(pl)) {
+        pl->sort_pending = 0;
         NB_CUDA(nb_launch_sort_by_length(pl, pl->len_key, true, s));
         pl->sorted = 1;
     }
@@ -413,11 +437,12 @@ static int forces_impl(const char *who, nb_pairlist *pl, int part, const float *
     const int kpart = split ? part : NB_PART_ALL;
     const bool last = part != NB_PART_LOCAL;  // this call ends the evaluation
     if (compute) {
-        NB_CUDA(sort_if_pending(pl, s));
+        const bool gathered = pl->has_vtiles && !(pl->flags & NB_FLAG_CLUSTER_TILES);
+        if (!gathered) NB_CUDA(sort_if_pending(pl, s));
         NB_CUDA(nb_launch_gather(pl, coords, q, type, ntype, 0, energies, kpart, s));
         if (pl->ev_start) NB_CUDA(cudaEventRecord(pl->ev_start, s));
         const int fpart = (!split && part == NB_PART_LOCAL) ? NB_PART_ALL : kpart;
-        if (pl->has_vtiles && !(pl->flags & NB_FLAG_CLUSTER_TILES))
+        if (gathered)
             NB_CUDA(nb_launch_force_vt(pl, ntype, ljparams, rc, beta, energies, stale_bound2(pl->r_inner, rc), fpart,
                                        s));
         else
@@ -463,7 +488,7 @@ extern "C" int nb_backward(nb_pairlist *pl, const float *coords, const float *q,
         return fail(NB_ERR_STATE, "nb_backward: NB_COUL_EXCL_CORR needs a search with exclusion lists made while it was set");
     DeviceGuard gd(pl->device);
     cudaStream_t s = (cudaStream_t)stream;
-    NB_CUDA(sort_if_pending(pl, s));
+    if (!pl->has_vtiles || (pl->flags & NB_FLAG_CLUSTER_TILES)) NB_CUDA(sort_if_pending(pl, s));
     NB_CUDA(nb_launch_gather_adj(pl, coords, q, type, ntype, g, s));
     NB_CUDA(nb_launch_backward(pl, ntype, ljparams, rc, beta, grad_x, grad_q, grad_lj, stale_bound2(pl->rlist, rc),
                                stale_bound2(pl->r_inner, rc), s));

@@ -457,7 +457,7 @@ static GatherParams gather_params(nb_pairlist *pl, const float *coords, const fl
     p.energies = energies;
     p.sys = pl->sys;
     p.clus_sys = pl->clus_sys;
-    p.len_hist = (snapshot && !(pl->flags & NB_FLAG_NO_LIST_SORT)) ? pl->len_hist : nullptr;
+    p.len_hist = snapshot && nb_prune_sorts(pl) ? pl->len_hist : nullptr;
     p.nsys = pl->nsys;
     p.snapshot = snapshot;
     return p;

@@ -122,8 +122,8 @@ struct nb_pairlist {
                           // clusters there are: captured searches make new ones, as many as their frame needs,
                           // without a call of the library, and captured force calls keep this address
     int sorted;           // an order by length was launched for the current list
-    int sort_pending;     // the last search's list is sorted by length at its first use (unless a prune
-                          // comes first and sorts its own)
+    int sort_pending;     // the current list is sorted by length at its use by a kernel over 8x8 tiles
+    int prune_captured;   // the last prune was captured: its replays make lists that the host does not see
     int *vt_slot;         // [2 cap * 8] gathered tiles: j slot | shift << 27
     unsigned *vt_mask;    // [2 cap] 4 x 8 in-range bits per gathered tile
     int *half_start;      // [2 parts][2 nc_max] first gathered tile of each half i-cluster
@@ -269,6 +269,12 @@ cudaError_t nb_launch_prune(nb_pairlist *pl, float r_inner2, float stale_search2
 // Orders i-clusters by decreasing ci_len. hist_ready: the histogram of
 // ci_len is already in len_hist (the prune computes it), else it is built here.
 cudaError_t nb_launch_sort_by_length(nb_pairlist *pl, const int *ci_len, bool hist_ready, cudaStream_t s);
+// Whether a prune orders the i-clusters of its list: only the kernels over 8x8 tiles take them in
+// that order (the three kernels: 4.5 us of a prune call of 18 to 23 us at 1,536 atoms). With
+// NB_FLAG_CLUSTER_TILES set later on, the calls that need the order make it (sort_if_pending).
+inline bool nb_prune_sorts(const nb_pairlist *pl) {
+    return !(pl->flags & NB_FLAG_NO_LIST_SORT) && (!pl->vt_slot || (pl->flags & NB_FLAG_CLUSTER_TILES));
+}
 // Clears the list-length histogram ahead of a prune that fills it.
 cudaError_t nb_clear_len_hist(nb_pairlist *pl, cudaStream_t s);
 // Records the excluded pairs of the caller's exclusion lists as slot pairs

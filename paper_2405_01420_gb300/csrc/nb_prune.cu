@@ -1,7 +1,7 @@
 // Rolling prune (§III-A, "Prune-only kernel"): outer list at rlist ->
 // inner list at r_inner, with atom-pair in-range masks. As in the paper's
 // post-pruning list sorting, the prune also computes the list-size
-// histogram that the sort needs.
+// histogram where a sort follows it (nb_prune_sorts).
 //
 // One warp per i-cluster (work counter). The outer entries are taken 32 at
 // a time, one per lane; the warp first stages the 32 j clusters in shared
@@ -356,7 +356,7 @@ cudaError_t nb_launch_prune(nb_pairlist *pl, float r_inner2, float stale_search2
     p.nl_list = pl->nl_list;
     p.pad_slot = pl->nc_max * NB_CLUSTER;
     p.len_key = pl->len_key;
-    p.len_hist = (pl->flags & NB_FLAG_NO_LIST_SORT) ? nullptr : pl->len_hist;
+    p.len_hist = nb_prune_sorts(pl) ? pl->len_hist : nullptr;
     p.r2cut = r_inner2;
     p.stale_search2 = stale_search2;
     // work_prune and inner_count were reset by the snapshot gather before this launch

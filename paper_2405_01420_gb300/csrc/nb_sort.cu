@@ -6,13 +6,11 @@
 // order of decreasing list length lets the longest lists start first, so the
 // persistent grid ends with short items and a short tail. For the kernels
 // over 8x8 tiles only: those over gathered tiles take the halves in cluster
-// order, in which half lists run from long to short already. A prune orders
-// its list all the same (3 us of a cycle of ten frames at 96,000 atoms):
-// NB_FLAG_CLUSTER_TILES may be set after it, and a call captured then, or one
-// over a replayed prune, could not make the order itself.
+// order, in which half lists run from long to short already.
 //
-// k_len_hist     histogram of the per-i-cluster list lengths (after a search;
-//                after a prune the prune kernel builds it, as in the paper)
+// k_len_hist     histogram of the per-i-cluster list lengths (of a list that
+//                the 8x8 kernels come to read; a prune that is to order its
+//                list builds it itself, as in the paper)
 // k_len_offsets  exclusive scan of the histogram from the longest length down
 // k_len_scatter  ci -> order[offset(len) + rank within its length]
 #include "nb_internal.cuh"

@@ -122,11 +122,13 @@ def test_eager_calls_over_a_captured_search(fr, prune, what, grow):
 
 @pytest.mark.parametrize("grow", [True, False])
 @pytest.mark.parametrize("what", ["forces", "backward"])
-@pytest.mark.parametrize("prune, sort_lists", [(True, True), (True, False), (False, True)])
-def test_a_captured_call_over_eager_searches(fr, prune, sort_lists, what, grow):
-    """An 8x8 call captured when its list had an order, replayed over later lists, ordered or not."""
+@pytest.mark.parametrize("prune, sort_lists, by_prune", [(True, True, True), (True, False, True), (False, True, True),
+                                                         (True, True, False)])
+def test_a_captured_call_over_eager_searches(fr, prune, sort_lists, by_prune, what, grow):
+    """An 8x8 call captured when its list had an order, or was to get it, replayed over later lists, ordered
+    or not."""
     first, second = fr.pair(grow)
-    pl = fr.nb.Pairlist(fr.n, cluster_tiles=True)
+    pl = fr.nb.Pairlist(fr.n, cluster_tiles=by_prune)
     x = first.clone()
 
     def lists():
@@ -135,7 +137,9 @@ def test_a_captured_call_over_eager_searches(fr, prune, sort_lists, what, grow):
             pl.prune(x, R_INNER)
 
     lists()
-    fr.call(pl, what, x)
+    if by_prune:
+        fr.call(pl, what, x)
+    pl.set_flags(cluster_tiles=True)
     F = torch.empty((fr.n, 3), device="cuda")
     graph, out = captured(lambda: fr.call(pl, what, x, F))
     graph.replay()

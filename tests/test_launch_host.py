@@ -1,7 +1,7 @@
 """Launch logic of the library on the host, over a stand-in CUDA runtime:
 a pair search one of whose launches fails leaves nothing behind that the next
-one would take for its own; a prune orders its list whichever kernels are to
-read it."""
+one would take for its own; calls over 8x8 tiles find their list's order, made
+by the prune or by themselves."""
 import ctypes
 
 import numpy as np
@@ -73,9 +73,11 @@ def test_a_failed_search_leaves_no_counts(lib, kernel, memset_fails_too):
     lib.nb_pairlist_destroy(pl)
 
 
-@pytest.mark.parametrize("capturing", [False, True])
+@pytest.mark.parametrize("capture", ["none", "calls", "prune"])
 @pytest.mark.parametrize("sort_lists", [True, False])
-def test_cluster_tiles_turned_on_after_a_prune_find_an_order(lib, sort_lists, capturing):
+def test_cluster_tiles_turned_on_after_a_prune_find_an_order(lib, sort_lists, capture):
+    """The first 8x8 call orders a list whose prune did not; every call does whose order would not outlive
+    it (captured) or whose list changes unseen (after a captured prune)."""
     from paper_2405_01420_gb300 import nb
     pl = create(lib)
     orders = []
@@ -85,20 +87,40 @@ def test_cluster_tiles_turned_on_after_a_prune_find_an_order(lib, sort_lists, ca
             orders.append(ctypes.cast(args[0], ctypes.POINTER(ctypes.c_void_p))[6])
 
     rec = fake_cuda.Recorder(lib, emulate)
-    assert lib.nb_set_flags(pl, 0 if sort_lists else nb.NB_FLAG_NO_LIST_SORT) == NB_OK
-    assert search(lib, pl, (3, 3, 3)) == NB_OK
+    no_sort = 0 if sort_lists else nb.NB_FLAG_NO_LIST_SORT
     x, q, t = np.zeros((N, 3), np.float32), np.zeros(N, np.float32), np.zeros(N, np.int32)
     lj, F = np.zeros((1, 1, 2), np.float32), np.zeros((N, 3), np.float32)
-    assert lib.nb_prune(pl, x.ctypes.data, 0.7, None) == NB_OK
-    assert any("k_len_scatter" in k for k in rec.names) == sort_lists
-    rec.names.clear()
-    lib.fake_capturing(capturing)
-    flags = nb.NB_FLAG_CLUSTER_TILES | (0 if sort_lists else nb.NB_FLAG_NO_LIST_SORT)
-    assert lib.nb_set_flags(pl, flags) == NB_OK
-    for _ in range(2):
+
+    def forces():
+        rec.names.clear()
         assert lib.nb_forces(pl, x.ctypes.data, q.ctypes.data, t.ctypes.data, 1, lj.ctypes.data, 0.6, 3.0,
                              F.ctypes.data, None, None) == NB_OK
+        return sum("k_len_scatter" in k for k in rec.names)
+
+    assert lib.nb_set_flags(pl, no_sort) == NB_OK
+    assert search(lib, pl, (3, 3, 3)) == NB_OK
+    lib.fake_capturing(capture == "prune")
+    assert lib.nb_prune(pl, x.ctypes.data, 0.7, None) == NB_OK
+    assert not any("k_len" in k for k in rec.names)
+    lib.fake_capturing(capture == "calls")
+    assert lib.nb_set_flags(pl, nb.NB_FLAG_CLUSTER_TILES | no_sort) == NB_OK
+    made = [forces() for _ in range(3)]
     lib.fake_capturing(False)
-    assert len(orders) == 2 and all((o is not None) == sort_lists for o in orders)
-    assert not any("k_len" in k for k in rec.names), "the order is the prune's"
+    made += [forces() for _ in range(2)]
+    want = {"none": [1, 0, 0, 0, 0], "calls": [1, 1, 1, 1, 0], "prune": [1, 1, 1, 1, 1]}[capture]
+    assert made == (want if sort_lists else [0] * 5)
+    assert [o is not None for o in orders] == [sort_lists] * 5
+    lib.nb_pairlist_destroy(pl)
+
+
+@pytest.mark.parametrize("cluster_tiles", [True, False])
+def test_a_prune_orders_the_list_that_8x8_kernels_read(lib, cluster_tiles):
+    from paper_2405_01420_gb300 import nb
+    pl = create(lib)
+    rec = fake_cuda.Recorder(lib)
+    assert lib.nb_set_flags(pl, nb.NB_FLAG_CLUSTER_TILES if cluster_tiles else 0) == NB_OK
+    assert search(lib, pl, (3, 3, 3)) == NB_OK
+    x = np.zeros((N, 3), np.float32)
+    assert lib.nb_prune(pl, x.ctypes.data, 0.7, None) == NB_OK
+    assert any("k_len_scatter" in k for k in rec.names) == cluster_tiles
     lib.nb_pairlist_destroy(pl)
