@@ -320,8 +320,10 @@ __global__ void __launch_bounds__(kPruneThreads, kPruneCtasPerSm) k_prune(PruneP
                 for (int r = 0; r < kSets; ++r) key += ntile[r];
                 atomicAdd(&s_total[1], (unsigned)key);
             }
-            p.len_key[ci] = key;
-            if (p.len_hist) atomicAdd(&p.len_hist[min(key, NB_LEN_BINS - 1)], 1);
+            if (p.len_hist) {
+                p.len_key[ci] = key;
+                atomicAdd(&p.len_hist[min(key, NB_LEN_BINS - 1)], 1);
+            }
         }
     }
     // the CTA's totals, from its last warp: two atomics per i-cluster on these addresses (with the

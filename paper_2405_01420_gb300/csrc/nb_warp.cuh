@@ -5,22 +5,10 @@
 
 #include <cuda_runtime.h>
 
-// cp.async of 16 / 4 bytes, global -> shared (cached in L1).
+// cp.async of 16 bytes, global -> shared (cached in L1).
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem) : "memory");
-}
-
-__device__ __forceinline__ void cp_async4(void *smem, const void *gmem) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(gmem) : "memory");
-}
-
-// cp.async of 4 bytes of which the first n (0 or 4) are read from gmem and
-// the rest are zero-filled; with n = 0 nothing is read.
-__device__ __forceinline__ void cp_async4_zfill(void *smem, const void *gmem, unsigned n) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(gmem), "r"(n) : "memory");
 }
 
 // Waits for this thread's outstanding cp.async copies.
