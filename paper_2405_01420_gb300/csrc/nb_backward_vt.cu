@@ -30,8 +30,9 @@ namespace {
 
 constexpr int kBvtThreads = 128;
 constexpr int kBvtWarps = kBvtThreads / 32;
-// 4 CTAs: up to 128 registers (123 used, no spills). The adjoint pass at 24,000 atoms: 101.5 us with the
-// j data staged by cp.async, a Horner erfcx and scalar LJ accumulators, 98.8 us as it is now.
+// 4 CTAs: up to 128 registers (all of them for Ewald, no spills). The force-matching step at 24,000 atoms
+// takes 75.9 us, 47 of them here (cold), issue and the FMA pipe at 48 and 47% of their cycles: latency (long
+// scoreboard 3.4 per issue) and the tail of 2.5 halves per warp.
 constexpr int kBvtCtasPerSm = 4;
 
 struct BvtParams {

@@ -147,7 +147,8 @@ __device__ __forceinline__ unsigned take_item(const VtParams &p, unsigned by_ind
 // computed, and group g + 2's slot words meanwhile.
 // Dynamic shared memory: the ntype x ntype LJ table, then per warp 3 float4
 // per j type (see s_lj2).
-// Bound by the FMA pipe and instruction issue together, each about 61% busy
+// Bound by the FMA pipe and instruction issue together, 64 and 61% busy at
+// 96,000 atoms without energies, 63 and 62% with them
 // (a packed instruction holds the pipe for 2 cycles), with 5 warps per
 // scheduler to cover a half's chain of dependent loads. RES x THREADS
 // resident threads per SM set the register cap; pick_shape says which is

@@ -270,7 +270,7 @@ cudaError_t nb_launch_prune(nb_pairlist *pl, float r_inner2, float stale_search2
 // ci_len is already in len_hist (the prune computes it), else it is built here.
 cudaError_t nb_launch_sort_by_length(nb_pairlist *pl, const int *ci_len, bool hist_ready, cudaStream_t s);
 // Whether a prune orders the i-clusters of its list: only the kernels over 8x8 tiles take them in
-// that order (the three kernels: 4.5 us of a prune call of 18 to 23 us at 1,536 atoms). With
+// that order (two kernels and the histogram: a prune call at 1,536 atoms 18.2 -> 22.5 us). With
 // NB_FLAG_CLUSTER_TILES set later on, the calls that need the order make it (sort_if_pending).
 inline bool nb_prune_sorts(const nb_pairlist *pl) {
     return !(pl->flags & NB_FLAG_NO_LIST_SORT) && (!pl->vt_slot || (pl->flags & NB_FLAG_CLUSTER_TILES));

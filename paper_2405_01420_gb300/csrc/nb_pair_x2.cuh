@@ -75,7 +75,7 @@ __device__ __forceinline__ float2 nb_erfcx_x2(float2 x) {
 // exp(-beta^2 r^2) in ex and erfc(beta r)/r in a, for forces and energies
 // alike. Forces need only c2b ex + a: the hardware's exp2 and one rational
 // for erfcx(x) + 2x/sqrt(pi) made calls without energies 9 to 15% faster
-// (11,997 atoms 19.0 -> 17.3 us, 96,000 84 -> 73, 1,000,002 827 -> 700), but
+// (11,997 atoms 19.5 -> 17.7 us, 96,000 84 -> 73, 1,000,002 823 -> 696), but
 // in FP32 that rational is off by up to 2.5e-7 where this form is by 1.3e-7,
 // the hardware's exp2 by 2^-22, and the forces' error against FP64 grew by
 // 1 to 5%.
